@@ -62,15 +62,15 @@ struct SimtParams {
 __device__ __forceinline__ float4 gen4_rk(int dist, const PhiloxRoundKeys& rk, uint32_t r,
                                           uint32_t c0) {
   if (dist == kRademacher) {
-    const uint4 x = rademacher_bits(rk, r, c0 >> 7, 0u);
+    const uint4 x = rademacher_bits(rk, r, c0 >> 7);
     const uint32_t wsel = (c0 >> 5) & 3u;
     const uint32_t w = wsel == 0 ? x.x : wsel == 1 ? x.y : wsel == 2 ? x.z : x.w;
     const uint32_t bits = w >> (c0 & 31u);
     return make_float4((bits & 1u) ? -1.f : 1.f, (bits & 2u) ? -1.f : 1.f,
                        (bits & 4u) ? -1.f : 1.f, (bits & 8u) ? -1.f : 1.f);
   }
-  if (dist == kUniform) return uniform4(rk, r, c0 >> 2, 0u);
-  return gaussian4(rk, r, c0 >> 2, 0u);
+  if (dist == kUniform) return uniform4(rk, r, c0 >> 2);
+  return gaussian4(rk, r, c0 >> 2);
 }
 
 // The generated values (t0 + t, l0 + l) of a stage, t < BT, l < BL, zero
@@ -328,7 +328,7 @@ __global__ void k_materialize(PhiloxKey key, int dist, int fmt, int scaled, floa
     const int64_t rr = i / cols, cc = i % cols;
     const uint32_t r = (uint32_t)(row0 + rr);
     const uint32_t c = (uint32_t)(col0 + cc);
-    const float4 v = gen4(dist, key, r, c & ~3u, 0u);
+    const float4 v = gen4(dist, key, r, c & ~3u);
     const uint32_t e = c & 3u;
     const float g = e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w;
     if (fmt == kFP32) {

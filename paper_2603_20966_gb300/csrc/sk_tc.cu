@@ -422,7 +422,7 @@ __device__ __forceinline__ void gen_stage(uint8_t* sdst, const ItemGeo& g, const
         const uint32_t c = static_cast<uint32_t>(cbase);  // a multiple of 32
         const uint32_t blk = c >> 7;
         if (blk != cached_blk[it]) {
-          words[it] = rademacher_bits(key, static_cast<uint32_t>(grow), blk, 0u);
+          words[it] = rademacher_bits(key, static_cast<uint32_t>(grow), blk);
           cached_blk[it] = blk;
         }
         const uint32_t wsel = (c >> 5) & 3u;
@@ -466,6 +466,12 @@ __device__ __forceinline__ void gen_stage(uint8_t* sdst, const ItemGeo& g, const
     const bool full = cbase + LK <= g.lend;
     const uint32_t j0 = static_cast<uint32_t>(cbase >> 2) + qd;  // Philox block, slab 0
     const int64_t row0 = g.p0 + rbase;
+    // the column parts of the two slabs serve all row passes, a row's part
+    // both slabs: 10 wide products for them per 8 tasks
+    PhiloxCol pc[KSTEPS];
+#pragma unroll
+    for (int slab = 0; slab < KSTEPS; ++slab)
+      pc[slab] = philox_col(key, j0 + 4u * static_cast<uint32_t>(slab));
     // two tasks in flight per thread: full unrolling of the 8 Philox +
     // Box-Muller tasks made the loop too large for the instruction cache
     // (11 % slower on the Gaussian sketch)
@@ -473,13 +479,12 @@ __device__ __forceinline__ void gen_stage(uint8_t* sdst, const ItemGeo& g, const
     for (int i = 0; i < NPASS; ++i) {
       const int64_t grow = row0 + static_cast<int64_t>(RSTEP) * i;
       const bool rv = grow < g.P;
+      const PhiloxRow pr = philox_row(key, static_cast<uint32_t>(grow));
 #pragma unroll
       for (int slab = 0; slab < KSTEPS; ++slab) {
         uint2 v = make_uint2(0u, 0u);
         if (rv && (full || cbase + 16 * slab + 4 * qd < g.lend)) {
-          const uint32_t j = j0 + 4u * static_cast<uint32_t>(slab);
-          const float4 a = DIST == kUniform ? uniform4(key, static_cast<uint32_t>(grow), j, 0u)
-                                            : gaussian4(key, static_cast<uint32_t>(grow), j, 0u);
+          const float4 a = entries4<DIST>(pr, pc[slab], key);
           v = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
         }
         *reinterpret_cast<uint2*>(sdst + slab * S_SLAB + off0 +
@@ -1580,6 +1585,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     u += it.nsteps;
     const int64_t g0 = it.g0, lend = it.lend;
     uint32_t cached_blk = 0xffffffffu;  // Philox words belong to one segment's rows
+    PhiloxRow prow[2];  // the row parts of this lane's two rows (Gaussian, uniform)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      prow[i] = philox_row(p.rk, static_cast<uint32_t>(g0 + gbase + 16 * wg + 8 * i + (lane & 7)));
     // this group's stages of the segment: g_item + s = grp (mod NGROUPS)
     const int g_item = g;
     for (int s = ((grp - g_item) % C::NGROUPS + C::NGROUPS) % C::NGROUPS; s < it.nsteps;
@@ -1612,7 +1621,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint32_t c = static_cast<uint32_t>(c0);
             const uint32_t blk = c >> 7;
             if (blk != cached_blk) {
-              words = rademacher_bits(p.rk, static_cast<uint32_t>(grow), blk, 0u);
+              words = rademacher_bits(p.rk, static_cast<uint32_t>(grow), blk);
               cached_blk = blk;
             }
             const uint32_t wsel = (c >> 5) & 3u;
@@ -1631,7 +1640,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // lanes of a store phase write 8 rows x 16 B: every bank once)
         const uint32_t qd = (static_cast<uint32_t>(lane) >> 3) & 3u;
         const bool cv = cbase + 4 * qd < lend;
-        const uint32_t j = static_cast<uint32_t>(cbase >> 2) + qd;  // Philox block
+        const PhiloxCol pc = philox_col(p.rk, static_cast<uint32_t>(cbase >> 2) + qd);
 #pragma unroll
         for (int it = 0; it < 2; ++it) {
           const int rr = 8 * it + (lane & 7);
@@ -1640,9 +1649,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int64_t grow = g0 + r;
           uint2 v = make_uint2(0u, 0u);
           if (grow < p.Q && cv) {
-            const float4 a = DIST == kUniform
-                                 ? uniform4(p.rk, static_cast<uint32_t>(grow), j, 0u)
-                                 : gaussian4(p.rk, static_cast<uint32_t>(grow), j, 0u);
+            const float4 a = entries4<DIST>(prow[it], pc, p.rk);
             v = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
           }
           const uint32_t off = kmaj_off(r, qd >> 1) + (qd & 1u) * 8u;
@@ -1756,7 +1763,10 @@ struct CfgQ {
   static constexpr uint32_t OFF_A = 0;
   static constexpr uint32_t OFF_S = OFF_A + NSO * OPA;
   static constexpr uint32_t OFF_EPI = OFF_S + NSO * OPS;  // epilogue transpose tiles
-  static constexpr uint32_t OFF_BAR = OFF_EPI + NUM_EPI_WARPS * EPI_TILE;
+  // Philox column parts of a stage's 32 quads, per worker warp
+  static constexpr uint32_t OFF_COL = OFF_EPI + NUM_EPI_WARPS * EPI_TILE;
+  static constexpr uint32_t COL_BYTES = QK / 4 * sizeof(PhiloxCol);
+  static constexpr uint32_t OFF_BAR = OFF_COL + NUM_WORK_WARPS * COL_BYTES;
   // per slot: A landed, operands ready, slot read by both pairs' MMAs, S rows
   // received from the partner CTA; then the accumulator and drain barriers
   static constexpr uint32_t NUM_BARS = 4 * NSO + 3;
@@ -2000,6 +2010,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const bool gfirst = wg == 0;  // registers the expected bytes and waits for them
     const uint32_t s_bytes = static_cast<uint32_t>(gq) * QK;  // from all four partner warps
     const int ngroups8 = gq / 8;
+    PhiloxCol* cols = reinterpret_cast<PhiloxCol*>(smem + C::OFF_COL +
+                                                   (warp - WARP_WORK0) * C::COL_BYTES);
     int pend = -1;  // a stage whose copy into this CTA was expected, not yet waited for
     for (int s = grp; s < nsteps; s += C::NGROUPS) {
       const int so = s % C::NSO;
@@ -2013,6 +2025,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         pend = s;
       }
       const int64_t cbase = lbeg + static_cast<int64_t>(s) * QK;  // a multiple of 128
+      if (DIST != kRademacher) {  // lane l: the column part of quad l, for all the warp's rows
+        __syncwarp();
+        cols[lane] = philox_col(p.rk, static_cast<uint32_t>(cbase >> 2) + lane);
+        __syncwarp();
+      }
       for (int rg = wg; rg < ngroups8; rg += C::GROUP_WARPS) {
         const uint32_t r8 = static_cast<uint32_t>(gbase + 8 * rg);  // first row of the group
         if (DIST == kRademacher) {
@@ -2025,7 +2042,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           int64_t nv = 0;
           if (grow < p.Q && cbase < lend) {
             w = rademacher_bits(p.rk, static_cast<uint32_t>(grow),
-                                static_cast<uint32_t>(cbase >> 7), 0u);
+                                static_cast<uint32_t>(cbase >> 7));
             nv = min(lend - cbase, static_cast<int64_t>(QK));
           }
           const uint32_t word = qc == 0 ? w.x : qc == 1 ? w.y : qc == 2 ? w.z : w.w;
@@ -2054,18 +2071,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           // fill its 128 contiguous bytes)
           const uint32_t r = r8 + (static_cast<uint32_t>(lane) >> 2);
           const int64_t grow = g0 + r;
+          const PhiloxRow prow = philox_row(p.rk, static_cast<uint32_t>(grow));
 #pragma unroll 2
           for (int b = 0; b < 8; ++b) {
             const uint32_t c = static_cast<uint32_t>(b) * 16u + (static_cast<uint32_t>(lane) & 3u) * 4u;
             const int64_t cc = cbase + c;
             uint32_t q = 0u;
             if (grow < p.Q && cc < lend) {
-              const float4 a = DIST == kUniform
-                                   ? uniform4(p.rk, static_cast<uint32_t>(grow),
-                                              static_cast<uint32_t>(cc >> 2), 0u)
-                                   : gaussian4(p.rk, static_cast<uint32_t>(grow),
-                                               static_cast<uint32_t>(cc >> 2), 0u);
-              q = e4m3x4(a);
+              q = e4m3x4(entries4<DIST>(prow, cols[4 * b + (lane & 3)], p.rk));
             }
             *reinterpret_cast<uint32_t*>(sdst + q8_off(r, c)) = q;
           }
