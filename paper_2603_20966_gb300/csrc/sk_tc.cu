@@ -1157,29 +1157,40 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // tile's k rows (the pair MMA splits N between the two CTAs).  Warp roles,
 // chains and bounded waits are those of the left kernel.
 //
-// One ring of stages: the TMA brings a stage's FP32 A tile [256 rows][16]
-// into the slot (64-byte swizzle), and the workers split it in place.  The
-// 512 bytes of an 8-row group of the FP32 tile become that group's K-major
-// BF16 core matrices, hi (256 bytes: 8 rows x 2 halves of 8 columns) then
-// lo, so a warp converts whole groups with no other warp involved, and the
-// MMA reads hi and lo with 512 bytes between 8-row groups.  With no separate
-// staging ring the slots are 20 KB and the ring is 8 stages deep, so up to
-// 128 KB of A per SM are in flight from HBM.  The kernel is persistent: as
+// One ring of stages: the TMA brings a stage's FP32 A tile [256 rows][32]
+// into the slot (128-byte swizzle), and the workers split it in place.  The
+// 1024 bytes of an 8-row group of the FP32 tile become that group's K-major
+// BF16 core matrices, hi (512 bytes: 4 of 8 rows x 8 columns) then lo, so a
+// warp converts whole groups with no other warp involved, and the MMA reads
+// hi and lo with 1 KB between 8-row groups.  With no separate staging ring
+// the slots are 40 KB and the ring is 4 stages deep, so up to 128 KB of A per
+// SM are in flight from HBM.  A stage is 32 columns of n: with 16 (8 slots of
+// 20 KB) every row of the copy was a 64-byte piece of DRAM and the barriers,
+// fences and commits of a stage came twice as
+// often: 65536 x 16384, k = 256 1.174 -> 1.072 ms, the Nystrom pair of a
+// 50,000 x 50,000 matrix, r = 500 5.44 -> 4.96 ms.  Two groups of 8 worker
+// warps instead of four of 4: 1.103 and 5.11 ms (the fences and waits of a
+// stage then stop half the workers at once).  The kernel is persistent: as
 // many clusters as can be resident each take an equal contiguous share of
 // the stages of all blocks, with ring slots,
 // barrier phases and chains counted across items, so the next item's copies
 // and S tiles are under way while the last chain of the previous one drains.
 // ---------------------------------------------------------------------------
+constexpr int RK = 32;               // contracted length per stage of the right kernel
+constexpr int RSTEPS = RK / BK;      // MMA K steps per right stage
+constexpr int RCHAIN = CHAIN / RSTEPS;  // right stages per accumulation chain
+
 struct CfgR {
   static constexpr int ROWS = 256;  // rows of A per CTA (two 128-row accumulators)
   static constexpr int NGROUPS = 4;
   static constexpr int GROUP_WARPS = NUM_WORK_WARPS / NGROUPS;
   static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
-  static constexpr int NS = 8;                        // stages in the ring
-  static constexpr uint32_t OPA = BK * ROWS * 4;      // FP32 A tile = its hi and lo halves
+  static constexpr int NS = 4;                        // stages in the ring
+  static constexpr uint32_t OPA = RK * ROWS * 4;      // FP32 A tile = its hi and lo halves
   static constexpr uint32_t ACC_A = OPA / 2;          // hi + lo of one 128-row accumulator
-  static constexpr uint32_t GROUP_A = 512;            // one 8-row group, FP32 = hi + lo
-  static constexpr uint32_t OPS = 128 * BK * 2;       // this CTA's half of the S tile
+  static constexpr uint32_t GROUP_A = 8 * RK * 4;     // one 8-row group, FP32 = hi + lo
+  static constexpr uint32_t GROUP_S = 8 * RK * 2;     // one 8-row group of the S tile
+  static constexpr uint32_t OPS = 128 * RK * 2;       // this CTA's half of the S tile
   static constexpr uint32_t OFF_A = 0;
   static constexpr uint32_t OFF_S = OFF_A + NS * OPA;
   // epilogue area per warp: two staging tiles of a TMA drain, or the
@@ -1199,6 +1210,15 @@ struct CfgR {
   static_assert(OPA % 1024 == 0 && OPS % 1024 == 0, "slots on 1 KB boundaries");
   static_assert(OFF_EPI % 1024 == 0 && EPI_BYTES >= EPI_TILE_R, "epilogue tiles");
 };
+
+// Operand layout of a right stage: K-major core matrices (8 rows x 8
+// columns, 128 bytes, row r at 16 r), the four of an 8-row group of the 32
+// columns one after another; groups GROUP_S apart (S) or, hi before lo,
+// GROUP_A apart (A).  One K step is two core matrices: 256 bytes.
+constexpr uint32_t R_KSTEP = 256;
+__device__ __forceinline__ uint32_t right_s_off(uint32_t row, uint32_t chunk) {
+  return (row >> 3) * CfgR::GROUP_S + chunk * 128u + (row & 7u) * 16u;
+}
 
 struct TcRightParams {
   float* part;      // partials [segments][P][Q] (a block's segments in order)
@@ -1348,10 +1368,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     it.m0 = (mb * 4 + cr) * C::ROWS;  // this CTA's rows of A
     it.q0 = qt * nq;                  // the pair's k rows
     it.g0 = it.q0 + static_cast<int64_t>(rank) * gh;  // this CTA's S rows
-    it.lbeg = static_cast<int64_t>(s0) * BK;
-    it.lend = min(p.L, static_cast<int64_t>(s1) * BK);
+    it.lbeg = static_cast<int64_t>(s0) * RK;
+    it.lend = min(p.L, static_cast<int64_t>(s1) * RK);
     it.nsteps = s1 - s0;
-    it.nchains = (it.nsteps + CHAIN - 1) / CHAIN;
+    it.nchains = (it.nsteps + RCHAIN - 1) / RCHAIN;
     return it;
   };
 
@@ -1401,7 +1421,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           }
           mbar_arrive_expect_tx(full_b(so), C::OPA);
           tma_load_2d(sbase + C::OFF_A + so * C::OPA, &tmapA,
-                      static_cast<int32_t>(it.lbeg + static_cast<int64_t>(s) * BK),
+                      static_cast<int32_t>(it.lbeg + static_cast<int64_t>(s) * RK),
                       static_cast<int32_t>(it.m0), full_b(so));
           issued = g + 1;
         }
@@ -1415,12 +1435,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     if (lane == 0 && leader) {
       const uint32_t idesc = idesc_bf16_f32(256u, static_cast<uint32_t>(nq));
       // The single issuing thread's bookkeeping per stage bounds this kernel
-      // (it issues 4 MMAs per 512 tensor cycles), so the slot, phase and
+      // (it issues 8 MMAs per 1024 tensor cycles), so the slot, phase and
       // chain are counted, not divided, and every operand descriptor is a
       // base descriptor plus offset / 16 in its low word (exact: all offsets
       // are multiples of 16 B and every operand lies below 256 KB).
       const uint64_t a_base = smem_desc(sbase + C::OFF_A, LBO, C::GROUP_A);
-      const uint64_t b_base = smem_desc(sbase + C::OFF_S, LBO, SBO);
+      const uint64_t b_base = smem_desc(sbase + C::OFF_S, LBO, C::GROUP_S);
       const uint32_t a_lo = static_cast<uint32_t>(a_base);
       const uint64_t a_hi = a_base & 0xFFFFFFFF00000000ull;
       const uint32_t b_lo = static_cast<uint32_t>(b_base);
@@ -1446,21 +1466,24 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
         tc_fence_after();
         const uint32_t a_slot = a_lo + static_cast<uint32_t>(so) * (C::OPA >> 4);
-        const uint64_t bdesc = b_hi | (b_lo + static_cast<uint32_t>(so) * (C::OPS >> 4));
+        const uint32_t b_slot = b_lo + static_cast<uint32_t>(so) * (C::OPS >> 4);
 #pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-          // hi (pass 0) or lo (pass 1) of accumulator j: 8-row groups 512 B apart
+        for (int ks = 0; ks < RSTEPS; ++ks) {
+          const uint64_t bdesc = b_hi | (b_slot + ks * (R_KSTEP >> 4));
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const uint64_t adesc =
-                a_hi | (a_slot + ((static_cast<uint32_t>(pass) * 256u +
-                                   static_cast<uint32_t>(j) * C::ACC_A) >> 4));
-            mma_bf16_pair(tmem + static_cast<uint32_t>(j * nq), adesc, bdesc, idesc,
-                          (!chain_start || pass > 0) ? 1u : 0u);
+          for (int pass = 0; pass < 2; ++pass) {
+            // hi (pass 0) or lo (pass 1, half a group further) of accumulator j
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              const uint64_t adesc =
+                  a_hi | (a_slot + ((ks * R_KSTEP + pass * (C::GROUP_A / 2) + j * C::ACC_A) >> 4));
+              mma_bf16_pair(tmem + static_cast<uint32_t>(j * nq), adesc, bdesc, idesc,
+                            (!chain_start || ks > 0 || pass > 0) ? 1u : 0u);
+            }
           }
         }
         mma_commit_pair_mask(empty_o(so), 0xF);  // all four CTAs wrote into the slot
-        if (in_chain == CHAIN - 1 || s == nsteps - 1) {  // the chain ends
+        if (in_chain == RCHAIN - 1 || s == nsteps - 1) {  // the chain ends
           mma_commit_pair_mask(acc_full, pair_mask);
           in_chain = 0;
           ++chain_no;
@@ -1566,16 +1589,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // ---- workers: this CTA's half of the S tile, and its 256 rows of A ----
     const int grp = (warp - WARP_WORK0) / C::GROUP_WARPS;
     const int wt = threadIdx.x - 32 * WARP_WORK0 - grp * C::GROUP_THREADS;
-    static_assert(C::GROUP_WARPS == 4, "16 generated rows per warp cover gq <= 64");
+    // generated rows per warp, whole 8-row groups (gq <= 64 rows in all)
+    constexpr int WROWS = 64 / C::GROUP_WARPS, WITS = WROWS / 8;
+    static_assert(WROWS % 8 == 0, "whole 8-row groups per warp");
     const int wg = wt >> 5;       // warp of the group
     const bool gfirst = wg == 0;  // registers the expected bytes and waits for them
-    // warp wg generates rows 16 wg .. 16 wg + 15 of this CTA's generated rows
-    // (whole 8-row groups: 256 contiguous bytes each in the K-major layout)
+    // warp wg generates rows WROWS wg, ... of this CTA's generated rows
+    // (whole 8-row groups: 512 contiguous bytes each in the K-major layout)
     // and copies them into the partner itself, so no barrier spans the group
-    const int wrows = max(0, min(16, gq - 16 * wg));
-    const uint32_t w_off = static_cast<uint32_t>(gbase + 16 * wg) * 32u;
-    const uint32_t w_bytes = static_cast<uint32_t>(wrows) * 32u;
-    const uint32_t s_bytes = static_cast<uint32_t>(gq) * 32u;  // from all four partner warps
+    const int wrows = max(0, min(WROWS, gq - WROWS * wg));
+    const uint32_t w_off = static_cast<uint32_t>(gbase + WROWS * wg) * (RK * 2);
+    const uint32_t w_bytes = static_cast<uint32_t>(wrows) * (RK * 2);
+    const uint32_t s_bytes = static_cast<uint32_t>(gq) * (RK * 2);  // from all partner warps
     uint4 words = make_uint4(0u, 0u, 0u, 0u);
     int pend = -1;  // a stage whose copy into this CTA was expected, not yet waited for
     int g = 0;      // stages of the earlier segments
@@ -1585,10 +1610,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     u += it.nsteps;
     const int64_t g0 = it.g0, lend = it.lend;
     uint32_t cached_blk = 0xffffffffu;  // Philox words belong to one segment's rows
-    PhiloxRow prow[2];  // the row parts of this lane's two rows (Gaussian, uniform)
+    PhiloxRow prow[WITS];  // the row parts of this lane's rows (Gaussian, uniform)
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-      prow[i] = philox_row(p.rk, static_cast<uint32_t>(g0 + gbase + 16 * wg + 8 * i + (lane & 7)));
+    for (int i = 0; i < WITS; ++i)
+      prow[i] =
+          philox_row(p.rk, static_cast<uint32_t>(g0 + gbase + WROWS * wg + 8 * i + (lane & 7)));
     // this group's stages of the segment: g_item + s = grp (mod NGROUPS)
     const int g_item = g;
     for (int s = ((grp - g_item) % C::NGROUPS + C::NGROUPS) % C::NGROUPS; s < it.nsteps;
@@ -1608,17 +1634,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (lane == 0) mbar_arrive_expect_tx(s_recv(so), s_bytes);
         pend = g;
       }
-      const int64_t cbase = it.lbeg + static_cast<int64_t>(s) * BK;
+      const int64_t cbase = it.lbeg + static_cast<int64_t>(s) * RK;
       if (DIST == kRademacher) {
-        // a lane: one row (16 wg + lane % 16) and one 8-column half (lane / 16)
-        if ((lane & 15) < wrows) {
-          const uint32_t r = static_cast<uint32_t>(gbase + 16 * wg + (lane & 15));
-          const uint32_t hh = static_cast<uint32_t>(lane >> 4);
+        // a lane: row lane % WROWS of the warp's and 8-column chunks
+        // lane / WROWS, + 32 / WROWS, ..., whose signs are in one Philox word
+        if ((lane % WROWS) < wrows) {
+          const uint32_t r = static_cast<uint32_t>(gbase + WROWS * wg + lane % WROWS);
           const int64_t grow = g0 + r;
-          const int64_t c0 = cbase + 8 * hh;
-          uint4 v = make_uint4(0u, 0u, 0u, 0u);
-          if (grow < p.Q && c0 < lend) {
-            const uint32_t c = static_cast<uint32_t>(c0);
+          uint32_t w = 0u;
+          if (grow < p.Q) {
+            const uint32_t c = static_cast<uint32_t>(cbase);  // a multiple of 32, below lend
             const uint32_t blk = c >> 7;
             if (blk != cached_blk) {
               words = rademacher_bits(p.rk, static_cast<uint32_t>(grow), blk);
@@ -1626,34 +1651,44 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
             const uint32_t wsel = (c >> 5) & 3u;
             const uint4 wv = words;
-            const uint32_t w = wsel == 0 ? wv.x : wsel == 1 ? wv.y : wsel == 2 ? wv.z : wv.w;
-            const uint32_t bits = w >> (c & 31u);
-            v.x = 0x3F803F80u | ((bits & 1u) << 15) | ((bits & 2u) << 30);
-            v.y = 0x3F803F80u | ((bits & 4u) << 13) | ((bits & 8u) << 28);
-            v.z = 0x3F803F80u | ((bits & 16u) << 11) | ((bits & 32u) << 26);
-            v.w = 0x3F803F80u | ((bits & 64u) << 9) | ((bits & 128u) << 24);
+            w = wsel == 0 ? wv.x : wsel == 1 ? wv.y : wsel == 2 ? wv.z : wv.w;
           }
-          *reinterpret_cast<uint4*>(sdst + kmaj_off(r, hh)) = v;
+#pragma unroll
+          for (int i = 0; i < WITS; ++i) {
+            const uint32_t kc = static_cast<uint32_t>(lane / WROWS + i * (32 / WROWS));
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (grow < p.Q && cbase + 8 * kc < lend) {
+              const uint32_t bits = w >> (8u * kc);
+              v.x = 0x3F803F80u | ((bits & 1u) << 15) | ((bits & 2u) << 30);
+              v.y = 0x3F803F80u | ((bits & 4u) << 13) | ((bits & 8u) << 28);
+              v.z = 0x3F803F80u | ((bits & 16u) << 11) | ((bits & 32u) << 26);
+              v.w = 0x3F803F80u | ((bits & 64u) << 9) | ((bits & 128u) << 24);
+            }
+            *reinterpret_cast<uint4*>(sdst + right_s_off(r, kc)) = v;
+          }
         }
       } else {
-        // a lane owns quad qd = lane / 8 of rows 16 wg + 8 it + lane % 8 (the 16
-        // lanes of a store phase write 8 rows x 16 B: every bank once)
+        // a lane owns quads qd and qd + 4 (qd = lane / 8) of rows
+        // WROWS wg + 8 it + lane % 8 (the 16 lanes of a store phase write
+        // 8 rows x 16 B: every bank once); two entries' chains in flight
         const uint32_t qd = (static_cast<uint32_t>(lane) >> 3) & 3u;
-        const bool cv = cbase + 4 * qd < lend;
-        const PhiloxCol pc = philox_col(p.rk, static_cast<uint32_t>(cbase >> 2) + qd);
+#pragma unroll (WITS == 1 ? 2 : 1)
+        for (uint32_t slab = 0; slab < RSTEPS; ++slab) {
+          const int64_t c = cbase + 16 * slab + 4 * qd;
+          const PhiloxCol pc = philox_col(p.rk, static_cast<uint32_t>(c >> 2));
 #pragma unroll
-        for (int it = 0; it < 2; ++it) {
-          const int rr = 8 * it + (lane & 7);
-          if (rr >= wrows) continue;
-          const uint32_t r = static_cast<uint32_t>(gbase + 16 * wg + rr);
-          const int64_t grow = g0 + r;
-          uint2 v = make_uint2(0u, 0u);
-          if (grow < p.Q && cv) {
-            const float4 a = entries4<DIST>(prow[it], pc, p.rk);
-            v = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+          for (int it = 0; it < WITS; ++it) {
+            const int rr = 8 * it + (lane & 7);
+            if (rr >= wrows) continue;
+            const uint32_t r = static_cast<uint32_t>(gbase + WROWS * wg + rr);
+            uint2 v = make_uint2(0u, 0u);
+            if (g0 + r < p.Q && c < lend) {
+              const float4 a = entries4<DIST>(prow[it], pc, p.rk);
+              v = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+            }
+            *reinterpret_cast<uint2*>(sdst + right_s_off(r, 2u * slab + (qd >> 1)) +
+                                      (qd & 1u) * 8u) = v;
           }
-          const uint32_t off = kmaj_off(r, qd >> 1) + (qd & 1u) * 8u;
-          *reinterpret_cast<uint2*>(sdst + off) = v;
         }
       }
       // this warp's rows are written: copy them into the partner (async
@@ -1668,28 +1703,27 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         stop = true;
         break;
       }
-      // split the FP32 A tile in place, two 8-row groups (512 bytes each) per
-      // warp at a time: lane = (group lane / 16, row r = lane % 8, columns
-      // 8 h .. 8 h + 7 with h = (lane / 8) % 2).  The TMA lands each 64-byte
-      // row with the 64-byte swizzle (16-byte unit u of row r at
-      // u ^ ((r / 2) mod 4)), so the 8 lanes of a load phase read 8 different
-      // bank groups; the row's hi core-matrix row (8 columns, 16 bytes)
-      // replaces bytes 128 h + 16 r of the group, its lo row 256 bytes
-      // further, so the 8 lanes of a store phase write 128 contiguous bytes
+      // split the FP32 A tile in place, one 8-row group (1 KB) per warp at a
+      // time: lane = (row r = lane % 8, columns 8 kc .. 8 kc + 7 with
+      // kc = lane / 8).  The TMA lands each 128-byte row with the 128-byte
+      // swizzle (16-byte unit u of row r at u ^ r), so the 8 lanes of a load
+      // phase read 8 different bank groups; the row's hi core-matrix row
+      // (8 columns, 16 bytes) replaces bytes 128 kc + 16 r of the group, its lo
+      // row 512 bytes further, so the 8 lanes of a store phase write 128
+      // contiguous bytes
       {
         uint8_t* slot = smem + C::OFF_A + so * C::OPA;
         const uint32_t r = static_cast<uint32_t>(lane) & 7u;
-        const uint32_t h = (static_cast<uint32_t>(lane) >> 3) & 1u;
-        const uint32_t sw = (r >> 1) & 3u;
-        const uint32_t ld0 = r * 64u + (((2u * h) ^ sw) << 4);
-        const uint32_t ld1 = r * 64u + (((2u * h + 1u) ^ sw) << 4);
-        const uint32_t dst = h * 128u + r * 16u;
+        const uint32_t kc = static_cast<uint32_t>(lane) >> 3;
+        const uint32_t ld0 = r * 128u + (((2u * kc) ^ r) << 4);
+        const uint32_t ld1 = r * 128u + (((2u * kc + 1u) ^ r) << 4);
+        const uint32_t dst = kc * 128u + r * 16u;
 #pragma unroll 2
-        for (int gi = 2 * wg + (lane >> 4); gi < C::ROWS / 8; gi += 2 * C::GROUP_WARPS) {
+        for (int gi = wg; gi < C::ROWS / 8; gi += C::GROUP_WARPS) {
           uint8_t* grp8 = slot + gi * C::GROUP_A;
           const float4 x = *reinterpret_cast<const float4*>(grp8 + ld0);
           const float4 y = *reinterpret_cast<const float4*>(grp8 + ld1);
-          __syncwarp();  // the warp's groups have been read
+          __syncwarp();  // the warp's group has been read
           const uint32_t h0 = pack_bf16x2(x.x, x.y), h1 = pack_bf16x2(x.z, x.w);
           const uint32_t h2 = pack_bf16x2(y.x, y.y), h3 = pack_bf16x2(y.z, y.w);
           // a - hi of two elements in one packed FMA (the product by -1 is
@@ -1703,7 +1737,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const float2 l3 = __ffma2_rn(f2(__uint_as_float(h3 << 16), __uint_as_float(h3 & 0xffff0000u)),
                                        f2(-1.0f, -1.0f), f2(y.z, y.w));
           *reinterpret_cast<uint4*>(grp8 + dst) = make_uint4(h0, h1, h2, h3);
-          *reinterpret_cast<uint4*>(grp8 + 256u + dst) =
+          *reinterpret_cast<uint4*>(grp8 + C::GROUP_A / 2 + dst) =
               make_uint4(pack_bf16x2(l0.x, l0.y), pack_bf16x2(l1.x, l1.y),
                          pack_bf16x2(l2.x, l2.y), pack_bf16x2(l3.x, l3.y));
         }
@@ -2828,7 +2862,7 @@ struct RightSegPlan {
 RightSegPlan plan_right_seg(const GemmShape& s) {
   RightSegPlan r;
   r.pl = plan_right(s);
-  r.steps = (s.L + BK - 1) / BK;
+  r.steps = (s.L + RK - 1) / RK;
   const int64_t blocks = r.pl.tiles_p / 4 * r.pl.tiles_q;
   r.units = blocks * r.steps;
   const int64_t resident = quad_slots() / 4;
@@ -2920,9 +2954,9 @@ cudaError_t tc_sketch_right(const sk_sketch* h, const GemmShape& s, const float*
   const RightSegPlan rs = plan_right_seg(s);
   const Plan& pl = rs.pl;
   CUtensorMap map;
-  // A[m x n]: n innermost; one box = 16 columns of n x 256 rows of m, each
-  // 64-byte row with the 64-byte swizzle (the in-place split's lane map)
-  if (!encode_map(&map, A, s.P, s.L, lda, BK, CfgR::ROWS, CU_TENSOR_MAP_SWIZZLE_64B))
+  // A[m x n]: n innermost; one box = 32 columns of n x 256 rows of m, each
+  // 128-byte row with the 128-byte swizzle (the in-place split's lane map)
+  if (!encode_map(&map, A, s.P, s.L, lda, RK, CfgR::ROWS, CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
   TcRightParams p;
   p.P = s.P;
