@@ -37,10 +37,12 @@ sk_status from_cuda(cudaError_t e) { return sk::status_from_cuda(e); }
 bool valid_dist(int d) { return d == SK_GAUSSIAN || d == SK_RADEMACHER || d == SK_UNIFORM; }
 bool valid_prec(int p) { return p == SK_FP32 || p == SK_BF16X2 || p == SK_FP8E4M3; }
 
-size_t workspace_for(const sk_sketch* h, const GemmShape& s) {
+// least: what a lent buffer has to hold (the tensor-core forms use some more
+// where they can)
+size_t workspace_for(const sk_sketch* h, const GemmShape& s, bool least = false) {
   if (h->prec == SK_FP32) return sk::simt_workspace_bytes(s);
   if (h->prec == SK_FP8E4M3) return s.left ? 0 : sk::q8_workspace_bytes(s);
-  return sk::tc_workspace_bytes(s);
+  return sk::tc_workspace_bytes(s, least);
 }
 
 // Make sure the handle has at least `need` bytes of scratch.
@@ -60,6 +62,12 @@ sk_status ensure_workspace(sk_sketch* h, size_t need) {
   h->ws = p;
   h->ws_bytes = need;
   return SK_OK;
+}
+
+// The scratch of an apply call; a lent buffer has to hold only the least.
+sk_status ensure_workspace(sk_sketch* h, const GemmShape& s) {
+  const bool lent = !h->ws_owned && h->ws != nullptr;
+  return ensure_workspace(h, workspace_for(h, s, lent));
 }
 
 sk_status check_apply(const sk_sketch* h, const float* A, int64_t m, int64_t n, int64_t lda,
@@ -92,7 +100,7 @@ sk_status apply(sk_sketch* h, const float* A, int64_t m, int64_t n, int64_t lda,
   }
   if (h->prec == SK_FP8E4M3 && ((reinterpret_cast<uintptr_t>(Y) & 15u) || ldy % 4 != 0))
     return SK_EINVAL;
-  st = ensure_workspace(h, workspace_for(h, s));
+  st = ensure_workspace(h, s);
   if (st != SK_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   cudaError_t e;
@@ -256,7 +264,7 @@ sk_status sk_apply_left_stored(sk_handle h, const void* S, int64_t lds, const fl
   s.L = m;
   st = sk::tc_check(s, A, lda, Y, ldy);
   if (st != SK_OK) return st;
-  st = ensure_workspace(h, workspace_for(h, s));
+  st = ensure_workspace(h, s);
   if (st != SK_OK) return st;
   return from_cuda(sk::tc_sketch_left_stored(h, s, S, lds, A, lda, Y, ldy, h->ws, h->ws_bytes,
                                              static_cast<cudaStream_t>(stream)));

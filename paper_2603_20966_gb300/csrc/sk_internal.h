@@ -64,9 +64,10 @@ cudaError_t simt_sketch(const sk_sketch* h, const GemmShape& s, const float* A, 
 cudaError_t materialize(const sk_sketch* h, int64_t row0, int64_t col0, int64_t rows,
                         int64_t cols, int fmt, int scaled, void* out, int64_t ld,
                         cudaStream_t st);
-// fixed-order reduction of split partials: Y[p*ldy+q] = scale * sum_z part[z][p][q]
-cudaError_t splitk_reduce(const float* part, int splits, int64_t P, int64_t Q, float scale,
-                          float* Y, int64_t ldy, cudaStream_t st);
+// fixed-order reduction of split partials, rows of ldp >= Q elements:
+// Y[p*ldy+q] = scale * sum_z part[z][p][q]
+cudaError_t splitk_reduce(const float* part, int splits, int64_t P, int64_t Q, int64_t ldp,
+                          float scale, float* Y, int64_t ldy, cudaStream_t st);
 
 // fixed-order reduction of many problems in one launch
 struct ReduceDesc {
@@ -139,7 +140,8 @@ cudaError_t batch_launch_members(const BatchMember* mbs, size_t count, int64_t i
                                  BatchArena* arena, cudaEvent_t ready, cudaStream_t st);
 
 // ---- BF16 split-A tensor-core form (sk_tc.cu) ----
-size_t tc_workspace_bytes(const GemmShape& s);
+// `least`: the bytes a lent buffer has to hold (partial rows without padding)
+size_t tc_workspace_bytes(const GemmShape& s, bool least = false);
 sk_status tc_check(const GemmShape& s, const float* A, int64_t lda, const float* Y, int64_t ldy);
 cudaError_t tc_sketch(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
                       float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st);

@@ -24,6 +24,20 @@ __device__ __forceinline__ void store_scaled(float* y, float scale, float4 v) {
                                               __fmul_rn(scale, v.z), __fmul_rn(scale, v.w));
 }
 
+// scale v into columns c .. c + W - 1 of a row of Y, those past Q left alone.
+template <int W, class V>
+__device__ __forceinline__ void store_columns(float* row, int64_t c, int64_t Q, float scale,
+                                              const V& v) {
+  if (c + W <= Q) {
+    store_scaled(row + c, scale, v);
+  } else {
+    const float* vv = reinterpret_cast<const float*>(&v);
+#pragma unroll
+    for (int u = 0; u < W; ++u)
+      if (c + u < Q) row[c + u] = __fmul_rn(scale, vv[u]);
+  }
+}
+
 // Adds `N` partials, all loaded before the first is added.
 template <int N, class V>
 __device__ __forceinline__ const float* add_run(V& s, const float* __restrict__ p,

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "sk_internal.h"
 #include "sk_reduce.cuh"
@@ -277,18 +278,16 @@ __global__ void __launch_bounds__(TPB, 1) k_sketch_fp32_simt(SimtParams p) {
 template <int W>
 __global__ void __launch_bounds__(256)
     k_splitk_reduce(const float* __restrict__ part, int splits, int64_t groups, int64_t gpr,
-                    float scale, float* __restrict__ Y, int64_t ldy) {
+                    int64_t Q, float scale, float* __restrict__ Y, int64_t ldy) {
+  using V = typename std::conditional<W == 4, float4, float>::type;
   const int64_t zstride = groups * W;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < groups;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = groups <= 0xffffffffLL
                           ? static_cast<int64_t>(static_cast<uint32_t>(i) / static_cast<uint32_t>(gpr))
                           : i / gpr;
-    float* y = Y + r * ldy + (i - r * gpr) * W;
-    if constexpr (W == 4)
-      store_scaled(y, scale, sum_partials<float4>(part + i * 4, zstride, splits));
-    else
-      store_scaled(y, scale, sum_partials<float>(part + i, zstride, splits));
+    store_columns<W>(Y + r * ldy, (i - r * gpr) * W, Q, scale,
+                     sum_partials<V>(part + i * W, zstride, splits));
   }
 }
 
@@ -308,14 +307,8 @@ __global__ void __launch_bounds__(256)
                           ? static_cast<int64_t>(static_cast<uint32_t>(i) / static_cast<uint32_t>(gpr))
                           : i / gpr;
     const int64_t c = (i - r * gpr) * 4;
-    const float4 v = sum_partials<float4>(d.part + i * 4, zstride, d.splits);
-    float* y = d.Y + r * d.ldy + c;
-    if (c + 4 <= d.Q) {
-      store_scaled(y, d.scale, v);
-    } else {
-      const float vv[4] = {v.x, v.y, v.z, v.w};
-      for (int u = 0; u < 4 && c + u < d.Q; ++u) y[u] = __fmul_rn(d.scale, vv[u]);
-    }
+    store_columns<4>(d.Y + r * d.ldy, c, d.Q, d.scale,
+                     sum_partials<float4>(d.part + i * 4, zstride, d.splits));
   }
 }
 
@@ -419,23 +412,25 @@ size_t simt_workspace_bytes(const GemmShape& s) {
   return sp > 1 ? (size_t)sp * (size_t)s.P * (size_t)s.Q * sizeof(float) : 0;
 }
 
-cudaError_t splitk_reduce(const float* part, int splits, int64_t P, int64_t Q, float scale,
-                          float* Y, int64_t ldy, cudaStream_t st) {
+cudaError_t splitk_reduce(const float* part, int splits, int64_t P, int64_t Q, int64_t ldp,
+                          float scale, float* Y, int64_t ldy, cudaStream_t st) {
   // 16-byte groups when the rows of both sides are whole groups and there are
   // enough of them to give every SM a block; below that, one element per
-  // thread spreads the loads over more SMs
-  const int64_t total = P * Q;
-  const bool vec = Q % 4 == 0 && ldy % 4 == 0 && reinterpret_cast<uintptr_t>(part) % 16 == 0 &&
-                   reinterpret_cast<uintptr_t>(Y) % 16 == 0 && total / 4 >= 256LL * num_sms();
-  const int64_t groups = vec ? total / 4 : total;
+  // thread spreads the loads over more SMs (partial rows padded past Q only
+  // go with the first)
+  const bool vec = ldp % 4 == 0 && ldy % 4 == 0 && reinterpret_cast<uintptr_t>(part) % 16 == 0 &&
+                   reinterpret_cast<uintptr_t>(Y) % 16 == 0 &&
+                   (ldp != Q || P * Q / 4 >= 256LL * num_sms());
+  const int64_t gpr = vec ? ldp / 4 : ldp;
+  const int64_t groups = P * gpr;
   const int threads = groups >= 256LL * num_sms() ? 256 : 64;
   const int64_t blocks = std::min<int64_t>((groups + threads - 1) / threads, 1LL << 20);
   if (vec)
-    k_splitk_reduce<4><<<(unsigned)blocks, threads, 0, st>>>(part, splits, groups, Q / 4, scale,
+    k_splitk_reduce<4><<<(unsigned)blocks, threads, 0, st>>>(part, splits, groups, gpr, Q, scale,
                                                              Y, ldy);
   else
-    k_splitk_reduce<1><<<(unsigned)blocks, threads, 0, st>>>(part, splits, groups, Q, scale, Y,
-                                                             ldy);
+    k_splitk_reduce<1><<<(unsigned)blocks, threads, 0, st>>>(part, splits, groups, gpr, Q, scale,
+                                                             Y, ldy);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -497,7 +492,7 @@ cudaError_t simt_sketch(const sk_sketch* h, const GemmShape& s, const float* A, 
   count_launches(1);
   e = cudaGetLastError();
   if (e != cudaSuccess || splits == 1) return e;
-  return splitk_reduce(static_cast<float*>(ws), splits, s.P, s.Q, h->scale, Y, ldy, st);
+  return splitk_reduce(static_cast<float*>(ws), splits, s.P, s.Q, s.Q, h->scale, Y, ldy, st);
 }
 
 cudaError_t materialize(const sk_sketch* h, int64_t row0, int64_t col0, int64_t rows,

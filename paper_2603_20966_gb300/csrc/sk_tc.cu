@@ -1221,8 +1221,9 @@ __device__ __forceinline__ uint32_t right_s_off(uint32_t row, uint32_t chunk) {
 }
 
 struct TcRightParams {
-  float* part;      // partials [segments][P][Q] (a block's segments in order)
+  float* part;      // partials [segments][P][ldp] (a block's segments in order)
   int64_t P, Q, L;  // P = m, Q = k, L = n
+  int64_t ldp;      // partial row stride, >= Q
   int nq;           // N of the MMA: k rows per pair tile (multiple of 16, <= 256)
   int tmem_cols;    // power of two >= 2 * nq
   PhiloxRoundKeys rk;
@@ -1508,7 +1509,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // chain stalls the MMA issuer, which waits for the whole TMEM).
     const int quarter = warp & 3;
     const int colset = (warp - WARP_EPI0) >> 2;
-    const bool vec_ok = (p.Q % 4) == 0;
+    const bool vec_ok = (p.ldp % 4) == 0;
     const int nchunk = (nq + 31) / 32;
     float* tile = reinterpret_cast<float*>(smem + C::OFF_EPI + (warp - WARP_EPI0) * C::EPI_BYTES);
     const int rsub = lane >> 3;       // row within a group of 4 (read side)
@@ -1558,7 +1559,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int64_t gm = grow0 + rr;
           const float4 a = *reinterpret_cast<const float4*>(tile + rr * C::EPI_PITCH_R + csub);
           if (gm < p.P && c < nq) {
-            float* d = p.part + (static_cast<int64_t>(it.z) * p.P + gm) * p.Q + col;
+            float* d = p.part + (static_cast<int64_t>(it.z) * p.P + gm) * p.ldp + col;
             if (vec_ok && col + 4 <= p.Q) {
               if (c0 == 0)
                 *reinterpret_cast<float4*>(d) = a;
@@ -2877,23 +2878,27 @@ RightSegPlan plan_right_seg(const GemmShape& s) {
 }
 
 // Y = scale x the sum, in segment order, of the partials of each element's
-// block (as many as segments the block was cut into).  W columns per thread;
-// a thread block is `txn` column groups x blockDim.x / txn rows and takes
-// every gridDim.x-th such row of the 1024-row block y, so a thread keeps its
-// columns (and their blocks' segment counts) for all its rows, and has the
-// loads of 4 rows in flight (before: one column per thread, one row in
-// flight, which left this pass waiting for the L2).  Bound by L2 and HBM
-// traffic.  Whole right sketches: 65536 x 16384, k = 256 1.210 -> 1.170 ms;
-// 20011 x 3071, k = 100 85 -> 69 us.
+// block (as many as segments the block was cut into).  W columns of a row per
+// thread (W = 4: partial rows of whole 16-byte units; Y's columns past Q are
+// not written); a thread block is `txn` column groups x blockDim.x / txn rows
+// and takes every gridDim.x-th such row of the 1024-row block y, so a thread
+// keeps its columns (and their blocks' segment counts) for all its rows.
+// Bound by L2 and HBM traffic once enough loads are in flight: 4 rows at a
+// time when blocks are cut into few segments, as for large problems (before
+// that, one column and one load per thread: whole right sketches of
+// 65536 x 16384, k = 256 1.210 -> 1.170 ms, 20011 x 3071, k = 100 85 ->
+// 69 us), 8 segments of one row at a time when into many, as for small ones
+// (2617 x 345, k = 167, 11 segments: 37 -> 18 us with the padded rows below).
+constexpr int kManySegments = 8;
 template <int W>
 __global__ void __launch_bounds__(256)
-    k_reduce_segments(const float* __restrict__ part, int64_t P, int64_t Q, int nq, int tiles_q,
-                      int64_t steps, int64_t units, int64_t ncl, float scale, int txn,
-                      float* __restrict__ Y, int64_t ldy) {
+    k_reduce_segments(const float* __restrict__ part, int64_t P, int64_t Q, int64_t ldp, int nq,
+                      int tiles_q, int64_t steps, int64_t units, int64_t ncl, float scale,
+                      int txn, float* __restrict__ Y, int64_t ldy) {
   using V = typename std::conditional<W == 4, float4, float>::type;
   constexpr int RU = 4;  // rows in flight per thread
-  const int64_t total = P * Q;
-  const int64_t gpr = Q / W;
+  const int64_t total = P * ldp;
+  const int64_t gpr = (Q + W - 1) / W;
   const int tx = static_cast<int>(threadIdx.x) % txn;
   const int ty = static_cast<int>(threadIdx.x) / txn;
   const int tyn = static_cast<int>(blockDim.x) / txn;
@@ -2901,43 +2906,66 @@ __global__ void __launch_bounds__(256)
   const int64_t mblocks = (P + 4 * CfgR::ROWS - 1) / (4 * CfgR::ROWS);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * tyn;
   for (int64_t mb = blockIdx.y; mb < mblocks; mb += gridDim.y) {
-    const int64_t r0 = mb * (4 * CfgR::ROWS);
-    const int64_t r1 = min(P, r0 + 4 * CfgR::ROWS);
+    const int64_t r0 = mb * (4 * CfgR::ROWS) + static_cast<int64_t>(blockIdx.x) * tyn + ty;
+    const int64_t r1 = min(P, (mb + 1) * (4 * CfgR::ROWS));
     for (int64_t g = tx; g < gpr; g += txn) {
       const int64_t c = g * W;
       const int64_t blk = mb * tiles_q + c / nq;
       const int nseg = static_cast<int>(seg_owner((blk + 1) * steps - 1, units, ncl) -
                                         seg_owner(blk * steps, units, ncl)) + 1;
-      for (int64_t r = r0 + static_cast<int64_t>(blockIdx.x) * tyn + ty; r < r1;
-           r += RU * stride) {
+      auto put = [&](int64_t r, const V& v) { store_columns<W>(Y + r * ldy, c, Q, scale, v); };
+      if (nseg >= kManySegments) {
+        for (int64_t r = r0; r < r1; r += stride)
+          put(r, sum_partials<V>(part + r * ldp + c, total, nseg));
+        continue;
+      }
+      for (int64_t r = r0; r < r1; r += RU * stride) {
         V acc[RU];
 #pragma unroll
         for (int u = 0; u < RU; ++u) set_zero(acc[u]);
-        for (int z = 0; z < nseg; ++z) {
-          V v[RU];
+        for (int z = 0; z < nseg; z += 2) {  // two segments of the rows in flight
+          V v[2][RU];
 #pragma unroll
-          for (int u = 0; u < RU; ++u)
-            if (r + u * stride < r1)
-              v[u] = *reinterpret_cast<const V*>(part + z * total + (r + u * stride) * Q + c);
+          for (int y = 0; y < 2; ++y)
 #pragma unroll
-          for (int u = 0; u < RU; ++u)
-            if (r + u * stride < r1) add_to(acc[u], v[u]);
+            for (int u = 0; u < RU; ++u)
+              if (z + y < nseg && r + u * stride < r1)
+                v[y][u] = *reinterpret_cast<const V*>(part + (z + y) * total +
+                                                      (r + u * stride) * ldp + c);
+#pragma unroll
+          for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int u = 0; u < RU; ++u)
+              if (z + y < nseg && r + u * stride < r1) add_to(acc[u], v[y][u]);
         }
 #pragma unroll
         for (int u = 0; u < RU; ++u)
-          if (r + u * stride < r1) store_scaled(Y + (r + u * stride) * ldy + c, scale, acc[u]);
+          if (r + u * stride < r1) put(r + u * stride, acc[u]);
       }
     }
   }
 }
 
-size_t tc_workspace_bytes(const GemmShape& s) {
+// Row stride of the partials: whole 16-byte units (the TMA drain and the
+// reduction's vector loads need them), or the bare row length q when the
+// workspace, lent by the caller, holds no more than that.  Bare rows that are
+// not whole units drain by scalar adds: left 48611 x 301, k = 602 took 139 us
+// with them, 101 us padded.
+int64_t padded_row(int64_t q) { return (q + 3) / 4 * 4; }
+int64_t partial_row(int64_t q, int64_t rows, size_t room) {
+  return static_cast<size_t>(rows) * static_cast<size_t>(padded_row(q)) * sizeof(float) <= room
+             ? padded_row(q)
+             : q;
+}
+
+size_t tc_workspace_bytes(const GemmShape& s, bool least) {
+  const int64_t row = least ? s.Q : padded_row(s.Q);
   if (s.left) {
     const LeftPlan pl = plan_left(s);
-    return split_bytes(s.L, s.Q) + static_cast<size_t>(pl.splits) * s.P * s.Q * sizeof(float);
+    return split_bytes(s.L, s.Q) + static_cast<size_t>(pl.splits) * s.P * row * sizeof(float);
   }
   const RightSegPlan rs = plan_right_seg(s);
-  return static_cast<size_t>(rs.zmax) * static_cast<size_t>(s.P) * static_cast<size_t>(s.Q) *
+  return static_cast<size_t>(rs.zmax) * static_cast<size_t>(s.P) * static_cast<size_t>(row) *
          sizeof(float);
 }
 
@@ -2972,7 +3000,8 @@ cudaError_t tc_sketch_right(const sk_sketch* h, const GemmShape& s, const float*
   p.part = static_cast<float*>(ws);
   CUtensorMap pmap;
   memset(&pmap, 0, sizeof(pmap));
-  p.tma_drain = encode_part_map(&pmap, p.part, s.P, s.Q, s.Q, rs.zmax) ? 1 : 0;
+  p.ldp = partial_row(s.Q, rs.zmax * s.P, ws_bytes);
+  p.tma_drain = encode_part_map(&pmap, p.part, s.P, s.Q, p.ldp, rs.zmax) ? 1 : 0;
   // persistent clusters of four CTAs, as many as can be resident, each
   // taking an equal contiguous share of the stages
   if (rs.units > (int64_t(1) << 31) - 1) return cudaErrorInvalidValue;  // 32-bit stage numbers
@@ -2992,21 +3021,22 @@ cudaError_t tc_sketch_right(const sk_sketch* h, const GemmShape& s, const float*
   if (e != cudaSuccess) return e;
   count_launches(1);
   const int64_t mblocks = pl.tiles_p / 4;  // blocks of 1024 rows of m
-  // 16-byte groups when the rows of the partials and of Y are whole groups
-  // (Y's alignment and ldy are the tensor-core forms' own conditions)
-  const bool vec = s.Q % 4 == 0;
-  const int64_t gpr = vec ? s.Q / 4 : s.Q;
+  const bool vec = p.ldp % 4 == 0;  // Y and ldy: the tensor-core forms' own conditions
+  const int64_t gpr = vec ? p.ldp / 4 : s.Q;
   const int txn = static_cast<int>(std::min<int64_t>(gpr, 256));
   const int tyn = 256 / txn;
-  const int64_t per = (4 * CfgR::ROWS + 4 * tyn - 1) / (4 * tyn);  // one pass of 4 rows a thread
-  const dim3 rgrid(static_cast<unsigned>(per),
+  // one pass: 4 rows a thread, or 1 of many segments
+  const int rows = tyn * (rs.zmax >= kManySegments ? 1 : 4);
+  const dim3 rgrid(static_cast<unsigned>((4 * CfgR::ROWS + rows - 1) / rows),
                    static_cast<unsigned>(std::min<int64_t>(mblocks, 65535)));
   if (vec)
-    k_reduce_segments<4><<<rgrid, 256, 0, st>>>(p.part, s.P, s.Q, pl.nt, p.tiles_q, rs.steps,
-                                                rs.units, rs.ncl, h->scale, txn, Y, ldy);
+    k_reduce_segments<4><<<rgrid, 256, 0, st>>>(p.part, s.P, s.Q, p.ldp, pl.nt, p.tiles_q,
+                                                rs.steps, rs.units, rs.ncl, h->scale, txn, Y,
+                                                ldy);
   else
-    k_reduce_segments<1><<<rgrid, 256, 0, st>>>(p.part, s.P, s.Q, pl.nt, p.tiles_q, rs.steps,
-                                                rs.units, rs.ncl, h->scale, txn, Y, ldy);
+    k_reduce_segments<1><<<rgrid, 256, 0, st>>>(p.part, s.P, s.Q, p.ldp, pl.nt, p.tiles_q,
+                                                rs.steps, rs.units, rs.ncl, h->scale, txn, Y,
+                                                ldy);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -3083,7 +3113,7 @@ cudaError_t q8_sketch_right_quantized(const sk_sketch* h, const GemmShape& s, co
   prof_mark(h->prof_stop, st);
   if (e != cudaSuccess) return e;
   count_launches(1);
-  return splitk_reduce(static_cast<float*>(part), pl.splits, s.P, s.Q, h->scale, Y, ldy, st);
+  return splitk_reduce(static_cast<float*>(part), pl.splits, s.P, s.Q, s.Q, h->scale, Y, ldy, st);
 }
 
 cudaError_t q8_sketch_right(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
@@ -3112,6 +3142,7 @@ cudaError_t tc_sketch_left(const sk_sketch* h, const GemmShape& s, const float* 
   const size_t sb = split_bytes(s.L, s.Q);
   const size_t need = sb + static_cast<size_t>(pl.splits) * s.P * s.Q * sizeof(float);
   if (ws == nullptr || ws_bytes < need) return cudaErrorInvalidValue;
+  const int64_t ldp = partial_row(s.Q, pl.splits * s.P, ws_bytes - sb);
   void* H = ws;
   float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + sb);
   sk_sketch* hm = const_cast<sk_sketch*>(h);
@@ -3127,7 +3158,7 @@ cudaError_t tc_sketch_left(const sk_sketch* h, const GemmShape& s, const float* 
   // Pair sketches split A inside the kernel where inline_split says so;
   // single CTAs and the stored-S mode read the halves the split pass writes
   const bool conv = S_stored == nullptr && inline_split(h->dist, pl) && fp32_map_ok(A, lda);
-  if (!fill_problem(&hs.probs[0], pl, s, H, part, h->seed, h->dist, conv ? A : nullptr, lda))
+  if (!fill_problem(&hs.probs[0], pl, s, H, part, h->seed, h->dist, conv ? A : nullptr, lda, ldp))
     return cudaErrorInvalidValue;
   if (S_stored && !encode_stored_map(&hs.probs[0].smap, S_stored, s.P, s.L, lds))
     return cudaErrorInvalidValue;
@@ -3155,7 +3186,7 @@ cudaError_t tc_sketch_left(const sk_sketch* h, const GemmShape& s, const float* 
   if (e != cudaSuccess) return e;
   count_launches(1);
   // fixed-order sum of the split partials, times 1/sqrt(k), into Y
-  return splitk_reduce(part, pl.splits, s.P, s.Q, h->scale, Y, ldy, st);
+  return splitk_reduce(part, pl.splits, s.P, s.Q, ldp, h->scale, Y, ldy, st);
 }
 
 }  // namespace
