@@ -180,8 +180,8 @@ sk_status sk_create(uint64_t seed, int dist, int64_t k, sk_handle* out) {
   h->wait_limit_ns = sk::kDefaultWaitLimitNs;
   h->stall_stage = -1;
   cudaError_t e = cudaGetDevice(&h->device);
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&h->d_status), sizeof(int) * 4);
-  if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int) * 4);
+  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&h->d_status), sk::kStatusBytes);
+  if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sk::kStatusBytes);
   if (e != cudaSuccess) {
     if (h->d_status) cudaFree(h->d_status);
     delete h;
@@ -356,7 +356,6 @@ sk_status sk_destroy(sk_handle h) {
   if (h->ws_owned && h->ws) cudaFree(h->ws);
   if (h->stage_A) cudaFree(h->stage_A);
   if (h->stage_Y) cudaFree(h->stage_Y);
-  if (h->d_sched) cudaFree(h->d_sched);
   if (h->d_status) cudaFree(h->d_status);
   delete h;
   return SK_OK;

@@ -13,7 +13,8 @@ struct sk_sketch {
   int prec;
   float scale;          // fl32(1/sqrt(k))
   int device;
-  int* d_status;        // device status word (sk_status values), 0 = OK
+  int* d_status;        // device status words [0..3] ([0] an sk_status, 0 = OK), then the
+                        // claim counter of the handle's left sketches [4]
   void* ws;             // split-K partials (owned or lent)
   size_t ws_bytes;
   bool ws_owned;
@@ -23,14 +24,12 @@ struct sk_sketch {
   size_t stage_Y_bytes;
   cudaEvent_t prof_start;  // optional measurement hook (caller-owned events)
   cudaEvent_t prof_stop;
-  void* d_sched;           // device copy of the tensor-core work list (problem + items)
-  size_t d_sched_bytes;
-  uint64_t sched_key[9];   // what the uploaded work list was built for
   uint64_t wait_limit_ns;  // limit of every bounded device wait (sk_debug_set_wait)
   int64_t stall_stage;     // injected stall of the tests (sk_debug_set_wait), or -1
 };
 
 namespace sk {
+constexpr size_t kStatusBytes = 8 * sizeof(int);  // of sk_sketch::d_status
 // Limit of a bounded device wait unless a test shortens it: far beyond any
 // healthy stage, short enough that a stuck kernel returns within seconds.
 constexpr uint64_t kDefaultWaitLimitNs = 2000000000ull;
@@ -43,6 +42,40 @@ void count_launches(uint64_t n);
 
 // sk_status of a CUDA error; remembers it for sk_last_cuda_error.
 sk_status status_from_cuda(cudaError_t e);
+
+// Waits until the kernel this one overlaps (launch_overlapped) has finished
+// and its writes are visible; returns at once after an ordinary launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next overlapped launch on the stream may begin (once every block of
+// this kernel has said so).
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A kernel launch that may begin while the kernel before it on the stream is
+// still running (programmatic dependent launch): every thread of `kernel`
+// calls pdl_wait() before it touches what that kernel reads or writes, which
+// waits until it has finished and its writes are visible.  What overlaps is
+// the launch and the kernel's prologue.  `cluster`: CTAs per cluster along x.
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, unsigned cluster, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // Record the handle's measurement-hook event, if any, on `st`.
 inline void prof_mark(cudaEvent_t ev, cudaStream_t st) {

@@ -281,6 +281,8 @@ __global__ void __launch_bounds__(256)
                     int64_t Q, float scale, float* __restrict__ Y, int64_t ldy) {
   using V = typename std::conditional<W == 4, float4, float>::type;
   const int64_t zstride = groups * W;
+  pdl_wait();
+  pdl_trigger();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < groups;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = groups <= 0xffffffffLL
@@ -297,6 +299,7 @@ __global__ void __launch_bounds__(256)
 // whole batch, against one column and one load in flight per thread.
 __global__ void __launch_bounds__(256)
     k_splitk_reduce_batched(const ReduceDesc* __restrict__ desc) {
+  pdl_wait();
   const ReduceDesc d = desc[blockIdx.y];
   const int64_t gpr = d.ldp / 4;
   const int64_t groups = d.P * gpr;
@@ -425,14 +428,9 @@ cudaError_t splitk_reduce(const float* part, int splits, int64_t P, int64_t Q, i
   const int64_t groups = P * gpr;
   const int threads = groups >= 256LL * num_sms() ? 256 : 64;
   const int64_t blocks = std::min<int64_t>((groups + threads - 1) / threads, 1LL << 20);
-  if (vec)
-    k_splitk_reduce<4><<<(unsigned)blocks, threads, 0, st>>>(part, splits, groups, gpr, Q, scale,
-                                                             Y, ldy);
-  else
-    k_splitk_reduce<1><<<(unsigned)blocks, threads, 0, st>>>(part, splits, groups, gpr, Q, scale,
-                                                             Y, ldy);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_overlapped(vec ? k_splitk_reduce<4> : k_splitk_reduce<1>, dim3((unsigned)blocks),
+                           dim3(threads), 0, st, 0, part, splits, groups, gpr, Q, scale, Y, ldy);
 }
 
 cudaError_t splitk_reduce_batched(const ReduceDesc* d_desc, int nprob, int64_t max_elems,
@@ -441,9 +439,9 @@ cudaError_t splitk_reduce_batched(const ReduceDesc* d_desc, int nprob, int64_t m
   int64_t bx = (max_elems / 4 + 255) / 256;
   if (bx > 64) bx = 64;
   if (bx < 1) bx = 1;
-  k_splitk_reduce_batched<<<dim3((unsigned)bx, (unsigned)nprob), 256, 0, st>>>(d_desc);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_overlapped(k_splitk_reduce_batched, dim3((unsigned)bx, (unsigned)nprob), dim3(256),
+                           0, st, 0, d_desc);
 }
 
 cudaError_t simt_sketch(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,

@@ -95,24 +95,24 @@ constexpr uint32_t EPI_TILE = 32 * EPI_PITCH * 4;
 constexpr uint32_t DRAIN_TILE = 32 * 32 * 4;
 
 // Per-CTA buffers of the left kernel.  A CTA of a pair holds NT/2 columns of
-// each split A tile.  NARROW (pairs only, batches whose tiles all have at most
-// 256 columns): half-width split A slots, so the operand ring is 8 stages
-// deep instead of 4.  TDRAIN (all but NARROW): each epilogue warp has two
-// 4 KB staging tiles from which the TMA adds a drained accumulator chain into
-// the partial (see drain_chain_tma); a narrow ring has no room for them.
+// each split A tile.  NARROW (launches whose tiles all have at most 256
+// columns): half-width split A slots, so the operand ring is 8 stages deep
+// instead of 4 on pairs, 4 instead of 2 on single CTAs.  TDRAIN (all but
+// narrow pairs): each epilogue warp has two 4 KB staging tiles from which the
+// TMA adds a drained accumulator chain into the partial (see
+// drain_chain_tma); a narrow pair's ring has no room for them.
 template <bool PAIR, bool NARROW = false>
 struct Cfg {
-  static_assert(PAIR || !NARROW, "narrow rings are a pair configuration");
-  static constexpr int COLS = NARROW ? NT_MAX / 4 : PAIR ? NT_MAX / 2 : NT_MAX;  // most A columns per CTA
+  static constexpr int COLS = NT_MAX / (PAIR ? 2 : 1) / (NARROW ? 2 : 1);  // most A columns per CTA
   // Worker groups take turns on successive stages.  A group that starts
   // stage s has finished stage s - NGROUPS, so waits never run more than one
   // barrier phase ahead (the parity test would alias) as long as
   // NGROUPS <= NSO.
-  static constexpr int NGROUPS = PAIR ? 4 : 2;
+  static constexpr int NGROUPS = PAIR || NARROW ? 4 : 2;
   static constexpr int GROUP_WARPS = NUM_WORK_WARPS / NGROUPS;
   static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
-  static constexpr int NSO = NARROW ? 8 : PAIR ? 4 : 2;     // operand stages
-  static constexpr bool TDRAIN = !NARROW;
+  static constexpr int NSO = (PAIR ? 4 : 2) * (NARROW ? 2 : 1);  // operand stages
+  static constexpr bool TDRAIN = !(PAIR && NARROW);
   static constexpr uint32_t OPB = 2u * COLS * LK * 2u;      // hi and lo tiles of a stage
   static constexpr uint32_t OPS = BM * LK * 2;              // S tile: KSTEPS slabs of 16
   static constexpr uint32_t OFF_B = 0;
@@ -187,21 +187,25 @@ struct LeftItem {
   int prob, tp, tq, z;
 };
 
-// Work list: every item of the launch, longest first.  Pairs (or single
-// CTAs) take the next unclaimed item from the device counter `claim` (zero
-// at launch) until the list is exhausted.
+// Work list.  A batch's items lie in device memory, longest first; a single
+// sketch (the kernel's own LeftProblem parameter) numbers its items
+// (z tiles_q + tq) tiles_p + tp, all equally long.  Pairs (or single CTAs)
+// take the next unclaimed item from the device counter `claim` (zero at
+// launch) until the list is exhausted; with `claim` null there are no more
+// items than pairs, and each takes the one of its own number without a queue.
 struct LeftSched {
-  const LeftProblem* probs;
-  const LeftItem* items;
+  const LeftProblem* probs;  // batches
+  const LeftItem* items;     // batches
   int* claim;
   int nitems;
+  int tiles_p, tiles_q;      // single sketches
   int* status;
   uint64_t timeout_ns;
   // failure-injection hook of the tests, -1 otherwise: the TMA producer
   // issues no copy for this stage (counted over each CTA's or pair's run),
   // so the waits that depend on it give up after timeout_ns
   long long stall_stage;
-  PhiloxRoundKeys rk;  // round keys of problem 0 (read when a launch has one distribution)
+  PhiloxRoundKeys rk;  // round keys of a single sketch
 };
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo_elem, float hi_elem) {
@@ -318,13 +322,26 @@ struct ItemGeo {
   int nsteps, nt, nmma, nh, bh, cols, dist;
   int chain;  // stages per accumulation chain
   int coff;   // stages by which this item's chain boundaries are shifted
+  int z;      // split (partial) of the item
 };
 
-template <bool PAIR>
-__device__ __forceinline__ ItemGeo item_geo(const LeftSched& sc, int idx, uint32_t rank) {
-  const LeftItem it = sc.items[idx];
+constexpr int kMixed = -1;
+constexpr int kStored = 3;
+
+// Item `idx` of a batch's list (DIST = kMixed), or of a single sketch.
+template <int DIST>
+__device__ __forceinline__ LeftItem left_item(const LeftSched& sc, int idx) {
+  if (DIST == kMixed) return sc.items[idx];
+  const int t = idx / sc.tiles_p;
+  return LeftItem{0, idx - t * sc.tiles_p, t % sc.tiles_q, t / sc.tiles_q};
+}
+
+template <int DIST, bool PAIR>
+__device__ __forceinline__ ItemGeo item_geo(const LeftSched& sc, const LeftProblem& one, int idx,
+                                            uint32_t rank) {
+  const LeftItem it = left_item<DIST>(sc, idx);
   ItemGeo g;
-  g.pr = sc.probs + it.prob;
+  g.pr = DIST == kMixed ? sc.probs + it.prob : &one;
   g.P = g.pr->P;
   g.key = g.pr->key;
   g.nt = g.pr->nt;
@@ -342,6 +359,7 @@ __device__ __forceinline__ ItemGeo item_geo(const LeftSched& sc, int idx, uint32
   // that the accumulator drains of concurrent pairs do not all reach L2 at
   // once; the shift is a function of the item alone, so the summation order
   // of a problem does not depend on what runs beside it.
+  g.z = it.z;
   g.chain = g.pr->chain;
   g.coff = ((it.tp * 7 + it.z * 13 + it.tq * 5) & 7) * (g.chain / 8);
   return g;
@@ -653,18 +671,17 @@ __device__ __noinline__ bool drain_chain_left(uint32_t tmem, int quarter, int co
 // kStored to read a caller-materialized BF16 S by TMA instead of generating
 // it (the "communicate Omega" side of the paper's Sec. 6.2 trade, for
 // measurement).
-constexpr int kMixed = -1;
-constexpr int kStored = 3;
-
-template <int DIST, bool PAIR, bool NARROW = false, bool ECONV = false>
+template <int DIST, bool PAIR, bool NARROW = false, bool EC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
-    k_sketch_bf16x2_left(const LeftSched sc) {
+    k_sketch_bf16x2_left(const __grid_constant__ LeftSched sc,
+                         const __grid_constant__ LeftProblem one) {
   using C = Cfg<PAIR, NARROW>;
-  // EC (pairs): the epilogue warps certify every stage's A tile to the MMA
-  // issuer, and split in place the FP32 tiles of Gaussian and uniform items
+  // EC: the epilogue warps certify every stage's A tile to the MMA issuer,
+  // and split in place the FP32 tiles of Gaussian and uniform items on pairs
   // (their workers are busy generating; the epilogue warps are idle between
-  // accumulator drains), so no split pass runs before those items
-  constexpr bool EC = ECONV && PAIR;
+  // accumulator drains) and of every item on single CTAs, so no split pass
+  // runs before those items
+  constexpr bool CONV = EC || (PAIR && (DIST == kRademacher || DIST == kMixed));
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -722,6 +739,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   if (PAIR) cluster_sync();  // the peer's barriers exist before any remote arrive
   tc_fence_after();
+  // what this launch reads and overwrites is ready once the one before it
+  // has finished; the reduction may set itself up beside this kernel
+  pdl_wait();
+  pdl_trigger();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, sc.status, sc.timeout_ns};
   // barriers of the even CTA, addressed from either CTA
@@ -729,8 +750,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t lead_acc_empty = PAIR ? mapa_shared(acc_empty, 0u) : acc_empty;
 
   // The even CTA's TMA producer claims item j of this pair and publishes it in
-  // both CTAs' queue slot (-1 once the list is exhausted).
+  // both CTAs' queue slot (-1 once the list is exhausted).  Without a claim
+  // counter every role knows its only item.
+  const bool fixed = sc.claim == nullptr;
+  auto fixed_item = [&](int j) -> int {
+    const int idx = static_cast<int>(blockIdx.x >> (PAIR ? 1 : 0));
+    return j == 0 && idx < sc.nitems ? idx : -1;
+  };
   auto produce_item = [&](int j) -> int {
+    if (fixed) return fixed_item(j);
     const int slot = j % IQ;
     if (j >= IQ && !mbar_wait(iq_empty(slot), ((j / IQ) & 1) ^ 1, ab, 0x18, j)) return -1;
     int idx = atomicAdd(sc.claim, 1);
@@ -746,6 +774,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // Every other role reads item j from its own CTA's slot (one thread per
   // role) and tells the producer the slot has been read.
   auto read_item = [&](int j) -> int {
+    if (fixed) return fixed_item(j);
     const int slot = j % IQ;
     if (!mbar_wait<true>(iq_full(slot), (j / IQ) & 1, ab, 0x19, j)) return -1;
     const int idx = *reinterpret_cast<volatile int*>(iq + slot);
@@ -768,9 +797,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int j = 0; !*abort_flag; ++j) {
         const int idx = leader ? produce_item(j) : read_item(j);
         if (idx < 0) break;
-        const ItemGeo ig = item_geo<PAIR>(sc, idx, rank);
+        const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
         const CUtensorMap* map = &ig.pr->map;
-        tma_prefetch_desc(map);
         if (DIST == kStored) tma_prefetch_desc(&ig.pr->smap);
         const uint32_t tx = static_cast<uint32_t>(2 * ig.cols * LK * 2) +  // hi + lo
                             (DIST == kStored ? C::OPS : 0u);               // + the S tile
@@ -778,10 +806,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             static_cast<int32_t>((ig.q0 + static_cast<int64_t>(rank) * ig.cols) / HCHUNK);
         // FP32 A, split in place by the workers (Rademacher items on pairs) or
         // by the epilogue warps (EC)
-        const bool conv =
-            (DIST == kRademacher || DIST == kMixed || EC) && PAIR && ig.pr->conv_inline;
+        const bool conv = CONV && ig.pr->conv_inline;
         const int32_t x0 = static_cast<int32_t>(ig.q0 + static_cast<int64_t>(rank) * ig.cols);
-        if (conv) tma_prefetch_desc(&ig.pr->amap);
+        tma_prefetch_desc(conv ? &ig.pr->amap : map);
         for (int s = 0; s < ig.nsteps; ++s, ++g) {
           const int so = g % C::NSO;
           // the MMAs that read this slot last time have completed
@@ -817,13 +844,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int j = 0; !stop; ++j) {
         const int idx = read_item(j);
         if (idx < 0) break;
-        const ItemGeo ig = item_geo<PAIR>(sc, idx, rank);
+        const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
         const uint32_t idesc =
             idesc_bf16_f32(PAIR ? 256u : 128u, static_cast<uint32_t>(ig.nh)) | IDESC_B_MN_MAJOR;
         // split A as loaded: [hi chunks][lo chunks] of 64 columns (4 KB each),
         // or, converted in place, [chunk][hi, lo] (8 KB per chunk)
-        const bool inl =
-            (DIST == kRademacher || DIST == kMixed || EC) && PAIR && ig.pr->conv_inline;
+        const bool inl = CONV && ig.pr->conv_inline;
         const uint32_t chunk_stride = inl ? 2 * HCHUNK_BYTES : HCHUNK_BYTES;
         const uint32_t pstride =
             inl ? HCHUNK_BYTES : static_cast<uint32_t>(ig.cols * LK * 2);  // hi -> lo tile
@@ -918,20 +944,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       int pend = -1;  // item whose chain ended at the last certified stage, or -1
       bool pend_first = false;
       auto drain_pending = [&]() -> bool {
-        const ItemGeo pg = item_geo<PAIR>(sc, pend, rank);
-        const LeftItem it = sc.items[pend];
+        const ItemGeo pg = item_geo<DIST, PAIR>(sc, one, pend, rank);
         if (C::TDRAIN && pg.pr->tma_drain)
-          return drain_chain_tma<PAIR>(tmem, quarter, colset, tile_u32, tile, pg, it.z,
+          return drain_chain_tma<PAIR>(tmem, quarter, colset, tile_u32, tile, pg, pg.z,
                                        pend_first, acc_full, lead_acc_empty, gc++, ab);
         float* part_item =
-            pg.pr->part + static_cast<int64_t>(it.z) * pg.pr->P * pg.pr->ldp + pg.q0;
+            pg.pr->part + static_cast<int64_t>(pg.z) * pg.pr->P * pg.pr->ldp + pg.q0;
         return drain_chain_left<PAIR>(tmem, quarter, colset, tile, pg, part_item, pend_first,
                                       acc_full, lead_acc_empty, gc++, ab);
       };
       for (int j = 0; !stop; ++j) {
         const int idx = read_item_warp(j);
         if (idx < 0) break;
-        const ItemGeo ig = item_geo<PAIR>(sc, idx, rank);
+        const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
         int chains = 0;  // chains of this item begun so far
         for (int s = 0; s < ig.nsteps; ++s, ++g) {
           const int so = g % C::NSO;
@@ -940,11 +965,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             stop = true;
             break;
           }
-          if (ig.pr->conv_inline && (DIST == kMixed ? ig.dist : DIST) != kRademacher)
+          if (ig.pr->conv_inline && (!PAIR || (DIST == kMixed ? ig.dist : DIST) != kRademacher))
             convert_stage(smem + C::OFF_B + so * C::OPB, ig.cols, cwt, cset, 2);
           fence_proxy_async_smem();  // the split tile is read by the tensor core
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(lead_full_o + 8u * so);
+          if (lane == 0) {
+            if (PAIR)
+              mbar_arrive_cluster(lead_full_o + 8u * so);
+            else
+              mbar_arrive(full_o(so));
+          }
           if (pend >= 0) {
             if (!drain_pending()) {
               stop = true;
@@ -968,15 +998,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int j = 0; !stop; ++j) {
         const int idx = read_item_warp(j);
         if (idx < 0) break;
-        const ItemGeo ig = item_geo<PAIR>(sc, idx, rank);
-        const LeftItem it = sc.items[idx];
+        const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
         const int64_t P = ig.pr->P, Q = ig.pr->Q, ldp = ig.pr->ldp;
-        float* part_item = ig.pr->part + static_cast<int64_t>(it.z) * P * ldp + ig.q0;
+        float* part_item = ig.pr->part + static_cast<int64_t>(ig.z) * P * ldp + ig.q0;
         const bool vec_ok = (ldp % 4) == 0;
         const int nchains = (ig.nsteps + ig.coff + ig.chain - 1) / ig.chain;
         if (C::TDRAIN && ig.pr->tma_drain) {
           for (int c0 = 0; c0 < nchains; ++c0) {
-            if (!drain_chain_tma<PAIR>(tmem, quarter, colset, tile_u32, tile, ig, it.z, c0 == 0,
+            if (!drain_chain_tma<PAIR>(tmem, quarter, colset, tile_u32, tile, ig, ig.z, c0 == 0,
                                        acc_full, lead_acc_empty, gc++, ab)) {
               stop = true;
               break;
@@ -1071,7 +1100,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int j = 0; !stop; ++j) {
       const int idx = read_item_warp(j);
       if (idx < 0) break;
-      const ItemGeo ig = item_geo<PAIR>(sc, idx, rank);
+      const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
 #pragma unroll
       for (int it = 0; it < RAD_IT; ++it) {  // Philox words belong to one problem and row
         cached_blk[it] = 0xffffffffu;
@@ -1405,6 +1434,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t partner_s = mapa_shared(sbase + C::OFF_S, partner);
   const uint32_t lead_acc_empty = mapa_shared(acc_empty, lead_rank);
   const uint16_t pair_mask = static_cast<uint16_t>(3u << (2u * pairi));
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == WARP_TMA) {
     if (lane == 0) {
@@ -1913,6 +1944,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t partner_s_recv = mapa_shared(s_recv(0), partner);
   const uint32_t partner_s = mapa_shared(sbase + C::OFF_S, partner);
   const uint16_t pair_mask = static_cast<uint16_t>(3u << (2u * pairi));
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == WARP_TMA) {
     if (lane == 0) {
@@ -2411,8 +2444,9 @@ LeftPlan plan_left(const GemmShape& s) {
   return pl;
 }
 
-// Whether a problem on pairs splits its FP32 A inside the sketch kernel.
-// Rademacher: always (the workers do it; their sign bits leave them idle).
+// Whether a problem splits its FP32 A inside the sketch kernel.  Single CTAs
+// (k <= 128: one tile of k): always, in the epilogue warps.  Rademacher on
+// pairs: always (the workers do it; their sign bits leave them idle).
 // Gaussian and uniform: the epilogue warps do it, once per 256-row pair tile
 // of k that reads the A tile, while the split pass splits it once; on the
 // 2^20 x 512, k = 2048 sketch (8 pair tiles) the in-kernel split cost 0.9 ms
@@ -2420,7 +2454,7 @@ LeftPlan plan_left(const GemmShape& s) {
 // most 4 pair tiles of k (k <= 1024) split A in the kernel.
 constexpr int64_t kInlineSplitMaxTiles = 4;
 bool inline_split(int dist, const LeftPlan& pl) {
-  return pl.pair && (dist == kRademacher || pl.tiles_p <= kInlineSplitMaxTiles);
+  return !pl.pair || dist == kRademacher || pl.tiles_p <= kInlineSplitMaxTiles;
 }
 
 // Split pass of one sketch (A rows 16-byte aligned, lda a multiple of 4).
@@ -2493,45 +2527,61 @@ void pack_sched(HostSched* hs) {
   memcpy(hs->blob.data() + hs->off_items, hs->items.data(), ib);
 }
 
-LeftSched device_sched(const HostSched& hs, void* dbuf, int* status,
-                       uint64_t timeout_ns = kDefaultWaitLimitNs, long long stall_stage = -1) {
+LeftSched device_sched(const HostSched& hs, void* dbuf, int* status) {
   LeftSched sc;
+  memset(&sc, 0, sizeof(sc));
   uint8_t* b = static_cast<uint8_t*>(dbuf);
   sc.probs = reinterpret_cast<const LeftProblem*>(b);
   sc.items = reinterpret_cast<const LeftItem*>(b + hs.off_items);
   sc.claim = reinterpret_cast<int*>(b + hs.off_claim);
   sc.nitems = static_cast<int>(hs.items.size());
   sc.status = status;
-  sc.timeout_ns = timeout_ns;
-  sc.stall_stage = stall_stage;
-  sc.rk = round_keys(hs.probs.empty() ? PhiloxKey{0u, 0u} : hs.probs[0].key);
+  sc.timeout_ns = kDefaultWaitLimitNs;
+  sc.stall_stage = -1;
   return sc;
 }
 
+// A batch's launch (its work list and claim counter in device memory) is an
+// ordinary one; a single sketch with no more items than pairs (claim null)
+// may begin while the kernel before it is still running.
 template <int DIST, bool PAIR, bool NARROW = false, bool EC = false>
-cudaError_t launch_left(const LeftSched& sc, int64_t units, cudaStream_t st) {
+cudaError_t launch_left(const LeftSched& sc, const LeftProblem& one, int64_t units,
+                        cudaStream_t st) {
   cudaError_t e = set_smem_attr<DIST, PAIR, NARROW, EC>();
   if (e != cudaSuccess) return e;
+  const dim3 grid(static_cast<unsigned>(units * (PAIR ? 2 : 1)), 1, 1);
+  if (sc.claim == nullptr)
+    return launch_overlapped(k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, grid, dim3(NTHREADS),
+                             Cfg<PAIR, NARROW>::SMEM, st, PAIR ? 2 : 1, sc, one);
   e = cudaMemsetAsync(sc.claim, 0, sizeof(int), st);  // the work list starts unclaimed
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  fill_config<PAIR>(&cfg, attr, dim3(static_cast<unsigned>(units * (PAIR ? 2 : 1)), 1, 1), st);
+  fill_config<PAIR>(&cfg, attr, grid, st);
   cfg.dynamicSmemBytes = Cfg<PAIR, NARROW>::SMEM;
-  return cudaLaunchKernelEx(&cfg, k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, sc);
+  return cudaLaunchKernelEx(&cfg, k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, sc, one);
+}
+
+template <int DIST, bool EC>
+cudaError_t launch_left_one(const LeftPlan& pl, const LeftSched& sc, const LeftProblem& one,
+                            int64_t units, cudaStream_t st) {
+  if (pl.pair) return launch_left<DIST, true, false, EC>(sc, one, units, st);
+  // single CTAs split A in the epilogue warps whatever S is (stored S apart)
+  constexpr bool SEC = DIST != kStored;
+  return pl.nt <= 256 ? launch_left<DIST, false, true, SEC>(sc, one, units, st)
+                      : launch_left<DIST, false, false, SEC>(sc, one, units, st);
 }
 
 // ec: Gaussian or uniform sketch on pairs whose A the epilogue warps split
-template <bool PAIR>
-cudaError_t launch_left_dist(int dist, const LeftSched& sc, int64_t units, cudaStream_t st,
-                             bool ec = false) {
-  if (dist == kStored) return launch_left<kStored, PAIR>(sc, units, st);
-  if (dist == kRademacher) return launch_left<kRademacher, PAIR>(sc, units, st);
+cudaError_t launch_left_dist(int dist, const LeftPlan& pl, const LeftSched& sc,
+                             const LeftProblem& one, int64_t units, cudaStream_t st, bool ec) {
+  if (dist == kStored) return launch_left_one<kStored, false>(pl, sc, one, units, st);
+  if (dist == kRademacher) return launch_left_one<kRademacher, false>(pl, sc, one, units, st);
   if (dist == kUniform)
-    return ec ? launch_left<kUniform, PAIR, false, PAIR>(sc, units, st)
-              : launch_left<kUniform, PAIR>(sc, units, st);
-  return ec ? launch_left<kGaussian, PAIR, false, PAIR>(sc, units, st)
-            : launch_left<kGaussian, PAIR>(sc, units, st);
+    return ec ? launch_left_one<kUniform, true>(pl, sc, one, units, st)
+              : launch_left_one<kUniform, false>(pl, sc, one, units, st);
+  return ec ? launch_left_one<kGaussian, true>(pl, sc, one, units, st)
+            : launch_left_one<kGaussian, false>(pl, sc, one, units, st);
 }
 
 // The split A of an m x n problem as a 4D tensor {64 columns, m rows,
@@ -2634,17 +2684,18 @@ bool encode_part_map(CUtensorMap* map, const float* part, int64_t P, int64_t Q, 
 }
 
 // A_inline: FP32 A (row stride lda) that the kernel splits in place instead
-// of reading the split pass's halves from H (problems on CTA pairs whose A
-// passes fp32_map_ok), or null.
+// of reading the split pass's halves from H (A has to pass fp32_map_ok), or
+// null.
 bool fill_problem(LeftProblem* pr, const LeftPlan& pl, const GemmShape& s, const void* H,
                   float* part, uint64_t seed, int dist, const float* A_inline = nullptr,
                   int64_t lda = 0, int64_t ldp = 0) {
   memset(pr, 0, sizeof(*pr));
-  if (!encode_split_map(&pr->map, H, s.L, s.Q, pl.pair ? pl.nt / 2 : pl.nt)) return false;
+  const int cols = pl.pair ? pl.nt / 2 : pl.nt;  // of a CTA
   if (A_inline != nullptr) {
-    if (!pl.pair) return false;
-    pr->conv_inline = encode_fp32_map(&pr->amap, A_inline, s.L, s.Q, lda, pl.nt / 2);
+    pr->conv_inline = encode_fp32_map(&pr->amap, A_inline, s.L, s.Q, lda, cols);
     if (pr->conv_inline == 0) return false;
+  } else if (!encode_split_map(&pr->map, H, s.L, s.Q, cols)) {
+    return false;
   }
   pr->part = part;
   pr->P = s.P;
@@ -2760,11 +2811,8 @@ cudaError_t launch_right_q(const CUtensorMap& map, const TcRightQParams& p, dim3
                            cudaStream_t st) {
   cudaError_t e = set_smem_attr_right_q();
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  fill_config<true>(&cfg, attr, grid, st, 4);
-  cfg.dynamicSmemBytes = CfgQ::SMEM;
-  return cudaLaunchKernelEx(&cfg, k_sketch_e4m3_right<DIST>, map, p);
+  return launch_overlapped(k_sketch_e4m3_right<DIST>, grid, dim3(NTHREADS), CfgQ::SMEM, st, 4, map,
+                           p);
 }
 
 // A_q[m x n] (row stride ldq bytes) as a 2D byte tensor; one box = 128 bytes
@@ -2804,11 +2852,8 @@ cudaError_t launch_right(const CUtensorMap& map, const CUtensorMap& pmap, const 
                          dim3 grid, cudaStream_t st) {
   cudaError_t e = set_smem_attr_right();
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  fill_config<true>(&cfg, attr, grid, st, 4);
-  cfg.dynamicSmemBytes = CfgR::SMEM;
-  return cudaLaunchKernelEx(&cfg, k_sketch_bf16x2_right<DIST>, map, pmap, p);
+  return launch_overlapped(k_sketch_bf16x2_right<DIST>, grid, dim3(NTHREADS), CfgR::SMEM, st, 4,
+                           map, pmap, p);
 }
 
 cudaError_t grow_device(void** buf, size_t* have, size_t need) {
@@ -2902,6 +2947,8 @@ __global__ void __launch_bounds__(256)
   const int tx = static_cast<int>(threadIdx.x) % txn;
   const int ty = static_cast<int>(threadIdx.x) / txn;
   const int tyn = static_cast<int>(blockDim.x) / txn;
+  pdl_wait();
+  pdl_trigger();
   if (ty >= tyn) return;
   const int64_t mblocks = (P + 4 * CfgR::ROWS - 1) / (4 * CfgR::ROWS);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * tyn;
@@ -3029,16 +3076,10 @@ cudaError_t tc_sketch_right(const sk_sketch* h, const GemmShape& s, const float*
   const int rows = tyn * (rs.zmax >= kManySegments ? 1 : 4);
   const dim3 rgrid(static_cast<unsigned>((4 * CfgR::ROWS + rows - 1) / rows),
                    static_cast<unsigned>(std::min<int64_t>(mblocks, 65535)));
-  if (vec)
-    k_reduce_segments<4><<<rgrid, 256, 0, st>>>(p.part, s.P, s.Q, p.ldp, pl.nt, p.tiles_q,
-                                                rs.steps, rs.units, rs.ncl, h->scale, txn, Y,
-                                                ldy);
-  else
-    k_reduce_segments<1><<<rgrid, 256, 0, st>>>(p.part, s.P, s.Q, p.ldp, pl.nt, p.tiles_q,
-                                                rs.steps, rs.units, rs.ncl, h->scale, txn, Y,
-                                                ldy);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_overlapped(vec ? k_reduce_segments<4> : k_reduce_segments<1>, rgrid, dim3(256), 0,
+                           st, 0, p.part, s.P, s.Q, p.ldp, pl.nt, p.tiles_q, rs.steps, rs.units,
+                           rs.ncl, h->scale, txn, Y, ldy);
 }
 
 int64_t q8_ld(int64_t n) { return (n + 15) / 16 * 16; }
@@ -3145,43 +3186,35 @@ cudaError_t tc_sketch_left(const sk_sketch* h, const GemmShape& s, const float* 
   const int64_t ldp = partial_row(s.Q, pl.splits * s.P, ws_bytes - sb);
   void* H = ws;
   float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + sb);
-  sk_sketch* hm = const_cast<sk_sketch*>(h);
-  // The work list depends only on these; upload it again only when they change.
-  const uint64_t key[9] = {reinterpret_cast<uint64_t>(A), static_cast<uint64_t>(s.L),
-                           static_cast<uint64_t>(s.Q), static_cast<uint64_t>(lda),
-                           reinterpret_cast<uint64_t>(ws), h->seed,
-                           static_cast<uint64_t>(h->dist) | (static_cast<uint64_t>(h->k) << 8),
-                           reinterpret_cast<uint64_t>(S_stored), static_cast<uint64_t>(lds)};
-  const int64_t units = pl.pair ? pair_slots() / 2 : num_sms_tc();
-  HostSched hs;
-  hs.probs.resize(1);
-  // Pair sketches split A inside the kernel where inline_split says so;
-  // single CTAs and the stored-S mode read the halves the split pass writes
+  const int64_t slots = pl.pair ? pair_slots() / 2 : num_sms_tc();
+  // A is split inside the kernel where inline_split says so; the others and
+  // the stored-S mode read the halves the split pass writes
   const bool conv = S_stored == nullptr && inline_split(h->dist, pl) && fp32_map_ok(A, lda);
-  if (!fill_problem(&hs.probs[0], pl, s, H, part, h->seed, h->dist, conv ? A : nullptr, lda, ldp))
+  LeftProblem pr;
+  if (!fill_problem(&pr, pl, s, H, part, h->seed, h->dist, conv ? A : nullptr, lda, ldp))
     return cudaErrorInvalidValue;
-  if (S_stored && !encode_stored_map(&hs.probs[0].smap, S_stored, s.P, s.L, lds))
+  if (S_stored && !encode_stored_map(&pr.smap, S_stored, s.P, s.L, lds))
     return cudaErrorInvalidValue;
-  build_items(std::vector<LeftPlan>{pl}, std::vector<int>{h->dist}, units, &hs);
-  pack_sched(&hs);
-  if (memcmp(key, hm->sched_key, sizeof(key)) != 0 || hm->d_sched_bytes < hs.bytes) {
-    cudaError_t e = grow_device(&hm->d_sched, &hm->d_sched_bytes, hs.bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(hm->d_sched, hs.blob.data(), hs.bytes, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
-    memcpy(hm->sched_key, key, sizeof(key));
-  }
-  const LeftSched sc = device_sched(hs, hm->d_sched, h->d_status, h->wait_limit_ns,
-                                    h->stall_stage);
-  const int64_t nunits = hs.units;
+  const int64_t items = pl.tiles_p * pl.tiles_q * pl.splits;
+  if (items > (int64_t(1) << 31) - 1) return cudaErrorInvalidValue;  // 32-bit item numbers
+  const int64_t units = std::max<int64_t>(1, std::min<int64_t>(slots, items));
+  LeftSched sc;
+  memset(&sc, 0, sizeof(sc));
+  sc.nitems = static_cast<int>(items);
+  sc.tiles_p = static_cast<int>(pl.tiles_p);
+  sc.tiles_q = static_cast<int>(pl.tiles_q);
+  sc.claim = items > units ? h->d_status + 4 : nullptr;
+  sc.status = h->d_status;
+  sc.timeout_ns = h->wait_limit_ns;
+  sc.stall_stage = h->stall_stage;
+  sc.rk = round_keys(pr.key);
   // the measurement hook brackets both passes: split of A (unless the kernel
   // splits it), then the sketch
   prof_mark(h->prof_start, st);
   cudaError_t e = conv ? cudaSuccess : split_launch_one(A, lda, s.L, s.Q, H, st);
   if (e != cudaSuccess) return e;
-  const int mode = S_stored ? kStored : h->dist;
-  e = pl.pair ? launch_left_dist<true>(mode, sc, nunits, st, conv && h->dist != kRademacher)
-              : launch_left_dist<false>(mode, sc, nunits, st);
+  e = launch_left_dist(S_stored ? kStored : h->dist, pl, sc, pr, units, st,
+                       conv && h->dist != kRademacher);
   prof_mark(h->prof_stop, st);
   if (e != cudaSuccess) return e;
   count_launches(1);
@@ -3384,11 +3417,13 @@ cudaError_t launch_plan(const PlannedBatch& pb, const BatchArena& ar, cudaStream
     count_launches(1);
   }
   const LeftSched sc = device_sched(pb.hs, ar.d_buf, ar.d_status);
+  LeftProblem none;
+  memset(&none, 0, sizeof(none));
   const cudaError_t e =
-      pb.narrow ? (pb.econv ? launch_left<kMixed, true, true, true>(sc, pb.units, st)
-                            : launch_left<kMixed, true, true>(sc, pb.units, st))
-                : (pb.econv ? launch_left<kMixed, true, false, true>(sc, pb.units, st)
-                            : launch_left<kMixed, true, false>(sc, pb.units, st));
+      pb.narrow ? (pb.econv ? launch_left<kMixed, true, true, true>(sc, none, pb.units, st)
+                            : launch_left<kMixed, true, true>(sc, none, pb.units, st))
+                : (pb.econv ? launch_left<kMixed, true, false, true>(sc, none, pb.units, st)
+                            : launch_left<kMixed, true, false>(sc, none, pb.units, st));
   if (e != cudaSuccess) return e;
   count_launches(1);
   return splitk_reduce_batched(reinterpret_cast<const ReduceDesc*>(b + pb.off_red),
