@@ -101,7 +101,15 @@ constexpr uint32_t DRAIN_TILE = 32 * 32 * 4;
 // narrow pairs): each epilogue warp has two 4 KB staging tiles from which the
 // TMA adds a drained accumulator chain into the partial (see
 // drain_chain_tma); a narrow pair's ring has no room for them.
-template <bool PAIR, bool NARROW = false>
+// SRING: the S tiles have a ring of their own, twice as deep as the A ring,
+// so a worker group that has handed a stage on starts its next one without
+// waiting for the MMAs of the first, and the workers go on through an
+// accumulator drain.  Each epilogue warp then has one staging tile instead of
+// two.  Left 2^20 x 512, k = 2048 Gaussian 4.278 -> 4.241 ms, batch of 256
+// 5.003 -> 4.982 ms: the workers are bound by the generator's instructions
+// (fused multiply-add pipe 62 % busy), not by slots; 20 of them at 64
+// registers instead of 16 at 72 made it 4.370 and 5.110 ms.
+template <bool PAIR, bool NARROW = false, bool SRING = false>
 struct Cfg {
   static constexpr int COLS = NT_MAX / (PAIR ? 2 : 1) / (NARROW ? 2 : 1);  // most A columns per CTA
   // Worker groups take turns on successive stages.  A group that starts
@@ -112,23 +120,26 @@ struct Cfg {
   static constexpr int GROUP_WARPS = NUM_WORK_WARPS / NGROUPS;
   static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
   static constexpr int NSO = (PAIR ? 4 : 2) * (NARROW ? 2 : 1);  // operand stages
+  static constexpr int NSS = SRING ? 8 : NSO;  // S tiles
   static constexpr bool TDRAIN = !(PAIR && NARROW);
+  static constexpr int STAGING = SRING ? 1 : 2;  // drain staging tiles per epilogue warp
   static constexpr uint32_t OPB = 2u * COLS * LK * 2u;      // hi and lo tiles of a stage
   static constexpr uint32_t OPS = BM * LK * 2;              // S tile: KSTEPS slabs of 16
   static constexpr uint32_t OFF_B = 0;
   static constexpr uint32_t OFF_S = OFF_B + NSO * OPB;
-  static constexpr uint32_t OFF_EPI = OFF_S + NSO * OPS;    // epilogue tiles, per warp:
-  static constexpr uint32_t EPI_BYTES = TDRAIN ? 2 * DRAIN_TILE : EPI_TILE;
+  static constexpr uint32_t OFF_EPI = OFF_S + NSS * OPS;    // epilogue tiles, per warp:
+  static constexpr uint32_t EPI_BYTES = TDRAIN ? STAGING * DRAIN_TILE : EPI_TILE;
   static constexpr uint32_t OFF_BAR = OFF_EPI + NUM_EPI_WARPS * EPI_BYTES;
-  static constexpr uint32_t NUM_BARS = 3 * NSO + 3 + 2 * IQ;
+  static constexpr uint32_t NUM_BARS = 2 * NSO + 2 * NSS + 3 + 2 * IQ;
   static constexpr uint32_t OFF_MISC = OFF_BAR + NUM_BARS * 8;  // abort flag, TMEM slot, item queue
   static constexpr uint32_t SMEM = OFF_MISC + 16 + 4 * IQ + 1024;  // + slack for 1 KB alignment
   // roles that read each queued item: in every CTA the epilogue and worker
   // warps, plus the MMA issuer (even CTA) or the TMA producer (odd CTA); the
   // even CTA's TMA producer fills the queue
+  // (a relay warp of the odd CTA, where there is one, comes on top)
   static constexpr int IQ_READERS = (PAIR ? 2 : 1) * (1 + NUM_EPI_WARPS + NUM_WORK_WARPS);
   static_assert(SMEM <= 227 * 1024, "shared memory budget");
-  static_assert(NGROUPS <= NSO, "worker groups vs ring depth");
+  static_assert(NGROUPS <= NSO && NSO <= NSS, "worker groups vs ring depths");
   static_assert(OPB % 1024 == 0, "split tiles start on swizzle-atom boundaries");
   static_assert(!TDRAIN || OFF_EPI % 1024 == 0, "staging tiles on swizzle-atom boundaries");
   static_assert(EPI_BYTES >= EPI_TILE, "the transpose tile fits the warp's area");
@@ -515,7 +526,7 @@ __device__ __forceinline__ void gen_stage(uint8_t* sdst, const ItemGeo& g, const
 // One accumulator drain by an epilogue warp of the left kernel through the
 // TMA: wait until chain gc has finished, and for each of the warp's 32-column
 // chunks of its TMEM lane quarter, read the chunk (lane = row), write it into
-// one of the warp's two staging tiles (row r at 128 r, its 16-byte unit u at
+// one of the warp's staging tiles (row r at 128 r, its 16-byte unit u at
 // u ^ (r mod 8): the 128-byte swizzle, and no bank conflict as the 8 lanes of
 // a phase write 8 different units), and let lane 0 hand the tile to the TMA,
 // which stores it into the item's partial (first chain) or adds it there
@@ -524,8 +535,8 @@ __device__ __forceinline__ void gen_stage(uint8_t* sdst, const ItemGeo& g, const
 // writes no longer hold up the next chain.  The adds of one address stay in
 // chain order, hence deterministic: lane 0 waits until its previous chain's
 // copies have completed before issuing this chain's, and a staging tile is
-// rewritten only after the copy two chunks back has read it.
-template <bool PAIR>
+// rewritten only after the copy STAGING chunks back has read it.
+template <bool PAIR, int STAGING>
 __device__ __noinline__ bool drain_chain_tma(uint32_t tmem, int quarter, int colset,
                                              uint32_t stage_u32, float* stage, const ItemGeo ig,
                                              int z, bool first, uint32_t acc_full,
@@ -551,9 +562,9 @@ __device__ __noinline__ bool drain_chain_tma(uint32_t tmem, int quarter, int col
     const int c = (ci * 32) & 255;
     const int tn =
         PAIR ? (c < ig.bh ? h * ig.bh + c : ig.cols + h * ig.bh + (c - ig.bh)) : ci * 32;
-    const uint32_t b = static_cast<uint32_t>(nb & 1);
-    if (nb >= 2) {
-      if (lane == 0) bulk_wait_read<1>();
+    const uint32_t b = static_cast<uint32_t>(nb % STAGING);
+    if (nb >= STAGING) {
+      if (lane == 0) bulk_wait_read<STAGING - 1>();
       __syncwarp();
     }
     float* row = stage + b * (DRAIN_TILE / 4) + lane * 32;
@@ -664,6 +675,14 @@ __device__ __noinline__ bool drain_chain_left(uint32_t tmem, int quarter, int co
   return true;
 }
 
+// Whether a launch runs the separate ring of S tiles (Cfg::SRING): the
+// wide pair kernels that generate Gaussian or uniform S.  Rademacher tiles
+// cost the workers little and their workers split A, so one ring of both
+// operands serves them; a stored S arrives with the A tile.
+template <int DIST, bool PAIR, bool NARROW>
+using LeftCfg =
+    Cfg<PAIR, NARROW, PAIR && !NARROW && (DIST == kGaussian || DIST == kUniform || DIST == kMixed)>;
+
 // Persistent left-sketch kernel: each pair (or single CTA) runs its list of
 // items back to back; ring positions, barrier phases and accumulation chains
 // are counted across items (g = stage counter, gc = chain counter).  DIST is
@@ -675,7 +694,10 @@ template <int DIST, bool PAIR, bool NARROW = false, bool EC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_sketch_bf16x2_left(const __grid_constant__ LeftSched sc,
                          const __grid_constant__ LeftProblem one) {
-  using C = Cfg<PAIR, NARROW>;
+  using C = LeftCfg<DIST, PAIR, NARROW>;
+  constexpr bool SRING = C::NSS > C::NSO;
+  // the odd CTA's second warp passes its landed A tiles on to the MMA issuer
+  constexpr bool RELAY = SRING && !EC;
   // EC: the epilogue warps certify every stage's A tile to the MMA issuer,
   // and split in place the FP32 tiles of Gaussian and uniform items on pairs
   // (their workers are busy generating; the epilogue warps are idle between
@@ -688,12 +710,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t sbase = smem_u32(smem);
   const uint32_t bar0 = sbase + C::OFF_BAR;
   // full_b: this CTA's split A tile has landed; full_o (even CTA): both CTAs'
-  // operands of the stage are ready; empty_o: the MMAs that read the slot
-  // have completed (signalled to both CTAs)
+  // operands of the stage are ready; empty_o: the MMAs of the stage have
+  // completed (signalled to both CTAs).  With a separate S ring full_o covers
+  // the S tiles (and what the workers split of A), full_a (even CTA) the A
+  // tiles the epilogue warps certify or, RELAY, the odd CTA's; empty_o
+  // counts stages in the S ring, so the slot of A that stage g reuses is free
+  // once barrier (g - NSO) mod NSS says so
   auto full_b = [&](int i) { return bar0 + 8u * i; };
   auto full_o = [&](int i) { return bar0 + 8u * (C::NSO + i); };
-  auto empty_o = [&](int i) { return bar0 + 8u * (2 * C::NSO + i); };
-  const uint32_t acc_full = bar0 + 8u * (3 * C::NSO);
+  auto empty_o = [&](int i) { return bar0 + 8u * (C::NSO + C::NSS + i); };
+  auto full_a = [&](int i) { return bar0 + 8u * (C::NSO + 2 * C::NSS + i); };
+  const uint32_t acc_full = bar0 + 8u * (2 * C::NSO + 2 * C::NSS);
   const uint32_t acc_empty = acc_full + 8u;
   const uint32_t drain_bar = acc_full + 16u;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
@@ -706,14 +733,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // item queue: slot i holds the index of the item every role of the pair
   // (or single CTA) works on next; iq_full / iq_empty: written / read by all
   int* iq = reinterpret_cast<int*>(smem + C::OFF_MISC + 16);
-  auto iq_full = [&](int i) { return bar0 + 8u * (3 * C::NSO + 3 + i); };
-  auto iq_empty = [&](int i) { return bar0 + 8u * (3 * C::NSO + 3 + IQ + i); };
+  auto iq_full = [&](int i) { return acc_full + 8u * (3 + i); };
+  auto iq_empty = [&](int i) { return acc_full + 8u * (3 + IQ + i); };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < C::NSO; ++i) {
       mbar_init(full_b(i), 1);
-      // one worker group of each CTA (plus, with EC, the epilogue warps of each)
-      mbar_init(full_o(i), (C::GROUP_WARPS + (EC ? NUM_EPI_WARPS : 0)) * (PAIR ? 2 : 1));
+      mbar_init(full_a(i), RELAY ? 1 : NUM_EPI_WARPS * 2);
+    }
+    for (int i = 0; i < C::NSS; ++i) {
+      // one worker group of each CTA (plus, with EC on one ring, the epilogue warps of each)
+      mbar_init(full_o(i), (C::GROUP_WARPS + (EC && !SRING ? NUM_EPI_WARPS : 0)) * (PAIR ? 2 : 1));
       mbar_init(empty_o(i), 1);
     }
     mbar_init(acc_full, 1);
@@ -721,7 +751,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     mbar_init(drain_bar, 1);
     for (int i = 0; i < IQ; ++i) {
       mbar_init(iq_full(i), 1);
-      mbar_init(iq_empty(i), C::IQ_READERS);
+      mbar_init(iq_empty(i), C::IQ_READERS + (RELAY ? 1 : 0));
     }
     *abort_flag = 0;
     mbar_fence_init();
@@ -747,6 +777,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const Abort ab{abort_flag, sc.status, sc.timeout_ns};
   // barriers of the even CTA, addressed from either CTA
   const uint32_t lead_full_o = PAIR ? mapa_shared(full_o(0), 0u) : full_o(0);
+  // where the epilogue warps (EC) certify A tiles, or the relay passes them on
+  const uint32_t lead_full_a = SRING ? mapa_shared(full_a(0), 0u) : lead_full_o;
   const uint32_t lead_acc_empty = PAIR ? mapa_shared(acc_empty, 0u) : acc_empty;
 
   // The even CTA's TMA producer claims item j of this pair and publishes it in
@@ -811,8 +843,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tma_prefetch_desc(conv ? &ig.pr->amap : map);
         for (int s = 0; s < ig.nsteps; ++s, ++g) {
           const int so = g % C::NSO;
-          // the MMAs that read this slot last time have completed
-          if (g >= C::NSO && !mbar_wait(empty_o(so), ((g / C::NSO) & 1) ^ 1, ab, 0x13, g)) break;
+          const int u = g - C::NSO;  // the stage that had this slot: its MMAs have completed
+          if (u >= 0 && !mbar_wait(empty_o(u % C::NSS), (u / C::NSS) & 1, ab, 0x13, g)) break;
           if (g == sc.stall_stage) continue;  // injected stall: this stage never lands
           mbar_arrive_expect_tx(full_b(so), tx);
           const int32_t y = static_cast<int32_t>(ig.lbeg + static_cast<int64_t>(s) * LK);
@@ -867,6 +899,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const uint64_t b_hi = b_base & 0xFFFFFFFF00000000ull;
         for (int s = 0; s < ig.nsteps; ++s, ++g) {
           const int so = g % C::NSO;
+          const int ss = g % C::NSS;
           const int ph = (s + ig.coff) & (ig.chain - 1);
           const bool chain_start = s == 0 || ph == 0;
           // a new chain may start only after every epilogue has read the last one
@@ -874,12 +907,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             stop = true;
             break;
           }
-          if (!mbar_wait(full_o(so), (g / C::NSO) & 1, ab, 0x22, g)) {
+          if ((SRING && !mbar_wait(full_a(so), (g / C::NSO) & 1, ab, 0x22, g)) ||
+              (RELAY && !mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x22, g)) ||
+              !mbar_wait(full_o(ss), (g / C::NSS) & 1, ab, 0x22, g)) {
             stop = true;
             break;
           }
           tc_fence_after();
-          const uint32_t a_slot = a_lo + ((static_cast<uint32_t>(so) * C::OPS) >> 4);
+          const uint32_t a_slot = a_lo + ((static_cast<uint32_t>(ss) * C::OPS) >> 4);
           const uint32_t b_slot = b_lo + ((static_cast<uint32_t>(so) * C::OPB) >> 4);
 #pragma unroll
           for (int ks = 0; ks < KSTEPS; ++ks) {
@@ -902,10 +937,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           }
           const bool chain_end = ph == ig.chain - 1 || s == ig.nsteps - 1;
           if (PAIR) {  // operands and accumulator are both CTAs'
-            mma_commit_pair_both(empty_o(so));
+            mma_commit_pair_both(empty_o(ss));
             if (chain_end) mma_commit_pair_both(acc_full);
           } else {
-            mma_commit(empty_o(so));
+            mma_commit(empty_o(ss));
             if (chain_end) mma_commit(acc_full);
           }
           if (chain_end) ++gc;
@@ -917,6 +952,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         mma_commit(drain_bar);
       // every MMA has finished before this CTA reaches the closing barrier
       drain_wait(drain_bar, 0, 200000000ull);
+    } else if (RELAY && lane == 0) {
+      int g = 0;
+      bool stop = false;
+      for (int j = 0; !stop; ++j) {
+        const int idx = read_item(j);
+        if (idx < 0) break;
+        const int nsteps = item_geo<DIST, PAIR>(sc, one, idx, rank).nsteps;
+        for (int s = 0; s < nsteps; ++s, ++g) {
+          const int so = g % C::NSO;
+          if (!mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x22, g)) {
+            stop = true;
+            break;
+          }
+          mbar_arrive_cluster(lead_full_a + 8u * so);
+        }
+      }
     }
   } else if (warp < WARP_WORK0) {
     // ---- epilogue: add each finished chain into the item's FP32 partial ----
@@ -946,7 +997,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       auto drain_pending = [&]() -> bool {
         const ItemGeo pg = item_geo<DIST, PAIR>(sc, one, pend, rank);
         if (C::TDRAIN && pg.pr->tma_drain)
-          return drain_chain_tma<PAIR>(tmem, quarter, colset, tile_u32, tile, pg, pg.z,
+          return drain_chain_tma<PAIR, C::STAGING>(tmem, quarter, colset, tile_u32, tile, pg, pg.z,
                                        pend_first, acc_full, lead_acc_empty, gc++, ab);
         float* part_item =
             pg.pr->part + static_cast<int64_t>(pg.z) * pg.pr->P * pg.pr->ldp + pg.q0;
@@ -971,7 +1022,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           __syncwarp();
           if (lane == 0) {
             if (PAIR)
-              mbar_arrive_cluster(lead_full_o + 8u * so);
+              mbar_arrive_cluster(lead_full_a + 8u * so);
             else
               mbar_arrive(full_o(so));
           }
@@ -1005,7 +1056,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int nchains = (ig.nsteps + ig.coff + ig.chain - 1) / ig.chain;
         if (C::TDRAIN && ig.pr->tma_drain) {
           for (int c0 = 0; c0 < nchains; ++c0) {
-            if (!drain_chain_tma<PAIR>(tmem, quarter, colset, tile_u32, tile, ig, ig.z, c0 == 0,
+            if (!drain_chain_tma<PAIR, C::STAGING>(tmem, quarter, colset, tile_u32, tile, ig, ig.z, c0 == 0,
                                        acc_full, lead_acc_empty, gc++, ab)) {
               stop = true;
               break;
@@ -1112,13 +1163,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
            s += C::NGROUPS) {
         g = g_item + s;
         const int so = g % C::NSO;
-        // the MMAs that read S tile `so` last time have completed
-        bool ok = g < C::NSO || mbar_wait(empty_o(so), ((g / C::NSO) & 1) ^ 1, ab, 0x43, g);
+        const int ss = g % C::NSS;
+        // the MMAs that read S tile `ss` last time have completed
+        bool ok = g < C::NSS || mbar_wait(empty_o(ss), ((g / C::NSS) & 1) ^ 1, ab, 0x43, g);
         if (!__all_sync(0xffffffffu, ok)) {  // leave together (abort path)
           stop = true;
           break;
         }
-        uint8_t* sdst = smem + C::OFF_S + so * C::OPS;
+        uint8_t* sdst = smem + C::OFF_S + ss * C::OPS;
         const int64_t cbase = ig.lbeg + static_cast<int64_t>(s) * LK;
         if constexpr (DIST == kStored) {
           // the S tile arrives with the split A tile
@@ -1137,7 +1189,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // leave them idle)
         const bool wconv = (DIST == kRademacher || DIST == kMixed) && PAIR &&
                            ig.pr->conv_inline && (DIST != kMixed || ig.dist == kRademacher);
-        if (!EC || wconv) {  // with EC the epilogue warps certify the A tile
+        if ((!EC && !SRING) || wconv) {  // otherwise the A tile is certified by others
           // this CTA's split A tile of the stage has landed
           ok = mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x40, g);
           if (!__all_sync(0xffffffffu, ok)) {
@@ -1153,9 +1205,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         __syncwarp();
         if (lane == 0) {
           if (PAIR)
-            mbar_arrive_cluster(lead_full_o + 8u * so);
+            mbar_arrive_cluster(lead_full_o + 8u * ss);
           else
-            mbar_arrive(full_o(so));
+            mbar_arrive(full_o(ss));
         }
       }
       g = g_item + ig.nsteps;
@@ -2310,7 +2362,7 @@ cudaError_t set_smem_attr() {
   if (done) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Cfg<PAIR, NARROW>::SMEM);
+                                       LeftCfg<DIST, PAIR, NARROW>::SMEM);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -2342,6 +2394,7 @@ int64_t pair_slots() {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_config<true>(&cfg, attr, dim3(2, 1, 1), nullptr);
+  cfg.dynamicSmemBytes = LeftCfg<kMixed, true, false>::SMEM;
   int clusters = 0;
   if (cudaOccupancyMaxActiveClusters(&clusters, k_sketch_bf16x2_left<kMixed, true>, &cfg) !=
           cudaSuccess ||
@@ -2552,13 +2605,13 @@ cudaError_t launch_left(const LeftSched& sc, const LeftProblem& one, int64_t uni
   const dim3 grid(static_cast<unsigned>(units * (PAIR ? 2 : 1)), 1, 1);
   if (sc.claim == nullptr)
     return launch_overlapped(k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, grid, dim3(NTHREADS),
-                             Cfg<PAIR, NARROW>::SMEM, st, PAIR ? 2 : 1, sc, one);
+                             LeftCfg<DIST, PAIR, NARROW>::SMEM, st, PAIR ? 2 : 1, sc, one);
   e = cudaMemsetAsync(sc.claim, 0, sizeof(int), st);  // the work list starts unclaimed
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_config<PAIR>(&cfg, attr, grid, st);
-  cfg.dynamicSmemBytes = Cfg<PAIR, NARROW>::SMEM;
+  cfg.dynamicSmemBytes = LeftCfg<DIST, PAIR, NARROW>::SMEM;
   return cudaLaunchKernelEx(&cfg, k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, sc, one);
 }
 
