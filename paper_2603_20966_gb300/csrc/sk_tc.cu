@@ -1244,8 +1244,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // BF16 core matrices, hi (512 bytes: 4 of 8 rows x 8 columns) then lo, so a
 // warp converts whole groups with no other warp involved, and the MMA reads
 // hi and lo with 1 KB between 8-row groups.  With no separate staging ring
-// the slots are 40 KB and the ring is 4 stages deep, so up to 128 KB of A per
-// SM are in flight from HBM.  A stage is 32 columns of n: with 16 (8 slots of
+// the slots are 32 KB and the ring is 4 stages deep, so up to 128 KB of A per
+// SM are in flight from HBM.  The S tiles have a ring of 8 of their own, so
+// a worker group generates its next S rows while the MMAs of its last stage
+// still read theirs and the A copy that waits for them is on its way
+// (0.993 -> 0.984 ms, Nystrom pair 4.74 -> 4.66 ms).  A stage is 32 columns of n: with 16 (8 slots of
 // 20 KB) every row of the copy was a 64-byte piece of DRAM and the barriers,
 // fences and commits of a stage came twice as
 // often: 65536 x 16384, k = 256 1.174 -> 1.072 ms, the Nystrom pair of a
@@ -1266,7 +1269,8 @@ struct CfgR {
   static constexpr int NGROUPS = 4;
   static constexpr int GROUP_WARPS = NUM_WORK_WARPS / NGROUPS;
   static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
-  static constexpr int NS = 4;                        // stages in the ring
+  static constexpr int NS = 4;                        // A tiles in the ring
+  static constexpr int NSS = 8;                       // S tiles
   static constexpr uint32_t OPA = RK * ROWS * 4;      // FP32 A tile = its hi and lo halves
   static constexpr uint32_t ACC_A = OPA / 2;          // hi + lo of one 128-row accumulator
   static constexpr uint32_t GROUP_A = 8 * RK * 4;     // one 8-row group, FP32 = hi + lo
@@ -1274,22 +1278,21 @@ struct CfgR {
   static constexpr uint32_t OPS = 128 * RK * 2;       // this CTA's half of the S tile
   static constexpr uint32_t OFF_A = 0;
   static constexpr uint32_t OFF_S = OFF_A + NS * OPA;
-  // epilogue area per warp: two staging tiles of a TMA drain, or the
-  // transpose tile (32 rows x 32 columns, pitch 36 floats) of the red.add one
-  static constexpr int EPI_PITCH_R = 36;
-  static constexpr uint32_t EPI_TILE_R = 32 * EPI_PITCH_R * 4;
-  static constexpr uint32_t EPI_BYTES = 2 * DRAIN_TILE;
-  static constexpr uint32_t OFF_EPI = OFF_S + NS * OPS;
+  // epilogue area per warp: the staging tile of a TMA drain, or the transpose
+  // tile of the red.add one (both 32 rows x 32 columns, swizzled)
+  static constexpr uint32_t EPI_BYTES = DRAIN_TILE;
+  static constexpr uint32_t OFF_EPI = OFF_S + NSS * OPS;
   static constexpr uint32_t OFF_BAR = OFF_EPI + NUM_EPI_WARPS * EPI_BYTES;
-  // per slot: A landed, operands ready, slot read by both pairs' MMAs, S rows
-  // received from the partner CTA; then the accumulator and drain barriers
-  static constexpr uint32_t NUM_BARS = 4 * NS + 3;
+  // per A slot: A landed, operands ready; per S slot: stage read by both
+  // pairs' MMAs, S rows received from the partner CTA; then the accumulator
+  // and drain barriers
+  static constexpr uint32_t NUM_BARS = 2 * NS + 2 * NSS + 3;
   static constexpr uint32_t OFF_MISC = OFF_BAR + NUM_BARS * 8;
   static constexpr uint32_t SMEM = OFF_MISC + 16 + 1024;
   static_assert(SMEM <= 227 * 1024, "shared memory budget");
-  static_assert(NGROUPS <= NS, "worker groups vs ring depth");
+  static_assert(NGROUPS <= NS && NS <= NSS, "worker groups vs ring depths");
   static_assert(OPA % 1024 == 0 && OPS % 1024 == 0, "slots on 1 KB boundaries");
-  static_assert(OFF_EPI % 1024 == 0 && EPI_BYTES >= EPI_TILE_R, "epilogue tiles");
+  static_assert(OFF_EPI % 1024 == 0, "epilogue tiles on swizzle-atom boundaries");
 };
 
 // Operand layout of a right stage: K-major core matrices (8 rows x 8
@@ -1356,12 +1359,11 @@ __device__ __noinline__ bool drain_right_tma(uint32_t tmem, int quarter, int col
                   static_cast<uint32_t>(j * nq + ci * 32),
               v);
     tmem_ld_wait();
-    const uint32_t b = static_cast<uint32_t>(nb & 1);
-    if (nb >= 2) {
-      if (lane == 0) bulk_wait_read<1>();
+    if (nb >= 1) {  // the TMA has read the previous chunk
+      if (lane == 0) bulk_wait_read<0>();
       __syncwarp();
     }
-    float* row = stage + b * (DRAIN_TILE / 4) + lane * 32;
+    float* row = stage + lane * 32;
 #pragma unroll
     for (int q = 0; q < 8; ++q)
       *reinterpret_cast<float4*>(row + ((static_cast<uint32_t>(q) ^ sw) << 2)) =
@@ -1372,11 +1374,10 @@ __device__ __noinline__ bool drain_right_tma(uint32_t tmem, int quarter, int col
     if (lane == 0) {
       const int32_t x = static_cast<int32_t>(q0 + ci * 32);
       const int32_t y = static_cast<int32_t>(m0 + j * 128 + quarter * 32);
-      const uint32_t src = stage_u32 + b * DRAIN_TILE;
       if (first)
-        tma_store_3d(pmap, src, x, y, z);
+        tma_store_3d(pmap, stage_u32, x, y, z);
       else
-        tma_reduce_add_3d(pmap, src, x, y, z);
+        tma_reduce_add_3d(pmap, stage_u32, x, y, z);
       bulk_commit();
     }
   }
@@ -1398,13 +1399,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t bar0 = sbase + C::OFF_BAR;
   // full_b: the slot's FP32 A tile has landed; full_o (even CTA): both CTAs'
   // operands of the stage are ready; empty_o: both pairs' MMAs have read
-  // what this CTA wrote into the slot (here and, S rows, in its partner);
-  // s_recv: the S rows the partner CTA copies into the slot have landed
+  // what this CTA wrote for the stage (here and, S rows, in its partner);
+  // s_recv: the S rows the partner CTA copies into the slot have landed.
+  // full_b and full_o count stages in the ring of A, the others in that of S
   auto full_b = [&](int i) { return bar0 + 8u * i; };
   auto full_o = [&](int i) { return bar0 + 8u * (C::NS + i); };
   auto empty_o = [&](int i) { return bar0 + 8u * (2 * C::NS + i); };
-  auto s_recv = [&](int i) { return bar0 + 8u * (3 * C::NS + i); };
-  const uint32_t acc_full = bar0 + 8u * (4 * C::NS);
+  auto s_recv = [&](int i) { return bar0 + 8u * (2 * C::NS + C::NSS + i); };
+  const uint32_t acc_full = bar0 + 8u * (2 * C::NS + 2 * C::NSS);
   const uint32_t acc_empty = acc_full + 8u;
   const uint32_t drain_bar = acc_full + 16u;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
@@ -1461,6 +1463,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int i = 0; i < C::NS; ++i) {
       mbar_init(full_b(i), 1);
       mbar_init(full_o(i), C::GROUP_WARPS * 2);  // one worker group of each CTA of the pair
+    }
+    for (int i = 0; i < C::NSS; ++i) {
       mbar_init(empty_o(i), 2);  // the MMAs of both pairs read what this CTA wrote
       mbar_init(s_recv(i), 1);   // the receiving group's expect-tx, plus the copy's bytes
     }
@@ -1498,8 +1502,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         u += it.nsteps;
         for (int s = 0; s < it.nsteps; ++s, ++g) {
           const int so = g % C::NS;
-          // both pairs' MMAs have read the slot's previous stage
-          if (g >= C::NS && !mbar_wait(empty_o(so), ((g / C::NS) & 1) ^ 1, ab, 0x13, g)) {
+          const int v = g - C::NS;  // the stage that had this slot: both pairs have read it
+          if (v >= 0 && !mbar_wait(empty_o(v % C::NSS), (v / C::NSS) & 1, ab, 0x13, g)) {
             stop = true;
             break;
           }
@@ -1529,7 +1533,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const uint64_t a_hi = a_base & 0xFFFFFFFF00000000ull;
       const uint32_t b_lo = static_cast<uint32_t>(b_base);
       const uint64_t b_hi = b_base & 0xFFFFFFFF00000000ull;
-      int so = 0, chain_no = 0, g = 0;
+      int so = 0, ss = 0, chain_no = 0, g = 0;
       uint32_t ph = 0;
       bool stop = false;
       for (int u = ubeg; u < uend && !stop;) {
@@ -1550,7 +1554,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
         tc_fence_after();
         const uint32_t a_slot = a_lo + static_cast<uint32_t>(so) * (C::OPA >> 4);
-        const uint32_t b_slot = b_lo + static_cast<uint32_t>(so) * (C::OPS >> 4);
+        const uint32_t b_slot = b_lo + static_cast<uint32_t>(ss) * (C::OPS >> 4);
 #pragma unroll
         for (int ks = 0; ks < RSTEPS; ++ks) {
           const uint64_t bdesc = b_hi | (b_slot + ks * (R_KSTEP >> 4));
@@ -1566,7 +1570,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
           }
         }
-        mma_commit_pair_mask(empty_o(so), 0xF);  // all four CTAs wrote into the slot
+        mma_commit_pair_mask(empty_o(ss), 0xF);  // all four CTAs wrote into the slot
         if (in_chain == RCHAIN - 1 || s == nsteps - 1) {  // the chain ends
           mma_commit_pair_mask(acc_full, pair_mask);
           in_chain = 0;
@@ -1578,6 +1582,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           so = 0;
           ph ^= 1u;
         }
+        if (++ss == C::NSS) ss = 0;
       }
       }
       mma_commit_pair(drain_bar);
@@ -1630,7 +1635,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // lane = accumulator row: its 32 columns into the tile
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4*>(tile + lane * C::EPI_PITCH_R + 4 * q) =
+          *reinterpret_cast<float4*>(tile + lane * 32 + 4 * (q ^ (lane & 7))) =
               make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
                           __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
         __syncwarp();
@@ -1640,7 +1645,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         for (int pass = 0; pass < 8; ++pass) {
           const int rr = 4 * pass + rsub;
           const int64_t gm = grow0 + rr;
-          const float4 a = *reinterpret_cast<const float4*>(tile + rr * C::EPI_PITCH_R + csub);
+          const float4 a =
+              *reinterpret_cast<const float4*>(tile + rr * 32 + (csub ^ (4 * (rr & 7))));
           if (gm < p.P && c < nq) {
             float* d = p.part + (static_cast<int64_t>(it.z) * p.P + gm) * p.ldp + col;
             if (vec_ok && col + 4 <= p.Q) {
@@ -1705,17 +1711,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
          s += C::NGROUPS) {
       g = g_item + s;
       const int so = g % C::NS;
-      // both pairs' MMAs have read what this CTA wrote into slot `so` (here
+      const int ss = g % C::NSS;
+      // both pairs' MMAs have read what this CTA wrote into S slot `ss` (here
       // and in its partner) last time
-      bool ok = g < C::NS || mbar_wait(empty_o(so), ((g / C::NS) & 1) ^ 1, ab, 0x43, g);
+      bool ok = g < C::NSS || mbar_wait(empty_o(ss), ((g / C::NSS) & 1) ^ 1, ab, 0x43, g);
       if (!__all_sync(0xffffffffu, ok)) {
         stop = true;
         break;
       }
-      uint8_t* sdst = smem + C::OFF_S + so * C::OPS;
+      uint8_t* sdst = smem + C::OFF_S + ss * C::OPS;
       // the partner's half of this CTA's S rows will land here
       if (gfirst) {
-        if (lane == 0) mbar_arrive_expect_tx(s_recv(so), s_bytes);
+        if (lane == 0) mbar_arrive_expect_tx(s_recv(ss), s_bytes);
         pend = g;
       }
       const int64_t cbase = it.lbeg + static_cast<int64_t>(s) * RK;
@@ -1780,8 +1787,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0 && w_bytes != 0)
-        bulk_copy_to_cluster(partner_s + static_cast<uint32_t>(so) * C::OPS + w_off,
-                             smem_u32(sdst) + w_off, w_bytes, partner_s_recv + 8u * so);
+        bulk_copy_to_cluster(partner_s + static_cast<uint32_t>(ss) * C::OPS + w_off,
+                             smem_u32(sdst) + w_off, w_bytes, partner_s_recv + 8u * ss);
       ok = mbar_wait(full_b(so), (g / C::NS) & 1, ab, 0x40, g);
       if (!__all_sync(0xffffffffu, ok)) {
         stop = true;
@@ -1829,7 +1836,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // the S half and the A operands are in this CTA's own shared memory;
       // the group's first warp certifies the partner's rows too
       fence_proxy_async_smem();
-      ok = !gfirst || mbar_wait(s_recv(so), (g / C::NS) & 1, ab, 0x46, g);
+      ok = !gfirst || mbar_wait(s_recv(ss), (g / C::NSS) & 1, ab, 0x46, g);
       if (!__all_sync(0xffffffffu, ok)) {
         stop = true;
         break;
@@ -1842,7 +1849,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
     // leaving early: let a copy the partner may still be sending land first
     if (gfirst && pend >= 0 && lane == 0)
-      drain_wait(s_recv(pend % C::NS), (pend / C::NS) & 1, 100000000ull);
+      drain_wait(s_recv(pend % C::NSS), (pend / C::NSS) & 1, 100000000ull);
   }
 
   tc_fence_before();
