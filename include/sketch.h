@@ -69,7 +69,10 @@ typedef enum {
 typedef enum { SK_GAUSSIAN = 0, SK_RADEMACHER = 1, SK_UNIFORM = 2 } sk_dist;
 
 /* Arithmetic form of the product.
- *  SK_FP32     FP32 generated operand, FP32 FMA on the CUDA cores.
+ *  SK_FP32     FP32 generated operand, products and sums of FP32 accuracy: right
+ *              sketches by FP32 FMA on the CUDA cores, left ones (of at least
+ *              64 rows) on the tensor cores with every FP32 operand as the
+ *              exact sum of three BF16 values.
  *  SK_BF16X2   generated operand rounded to BF16, A split into BF16 hi + lo
  *              parts (hi = bf16(a), lo = bf16(a - hi)), two tensor-core MMAs
  *              per tile with FP32 accumulation in tensor memory.

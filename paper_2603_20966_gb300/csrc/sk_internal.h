@@ -114,6 +114,12 @@ struct ReduceDesc {
 cudaError_t splitk_reduce_batched(const ReduceDesc* d_desc, int nprob, int64_t max_elems,
                                   cudaStream_t st);
 
+// ---- FP32 form of the left sketch on the tensor cores (sk_tc32.cu) ----
+bool tc32_applies(const GemmShape& s);
+size_t tc32_workspace_bytes(const GemmShape& s);
+cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
+                             float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st);
+
 // ---- batches of left sketches on the tensor cores (sk_tc.cu) ----
 struct BatchMember {
   uint64_t seed;

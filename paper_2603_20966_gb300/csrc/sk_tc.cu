@@ -64,6 +64,20 @@
 #include "sk_tc.cuh"
 
 namespace sk {
+
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  if (fn == nullptr) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault,
+                                         &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
+  }
+  return fn;
+}
+
 namespace {
 
 using namespace tc;
@@ -222,15 +236,6 @@ struct LeftSched {
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo_elem, float hi_elem) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo_elem, hi_elem);
   return *reinterpret_cast<uint32_t*>(&v);
-}
-
-// Bounded wait that ignores the abort flag (used only to drain in-flight
-// asynchronous work on the way out).
-__device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
-  const uint64_t t0 = globaltimer();
-  while (!mbar_try_wait(bar, parity)) {
-    if (globaltimer() - t0 > limit_ns) return;
-  }
 }
 
 // ---- split pass: A (FP32) -> hi / lo (BF16), rows padded to 64 columns ----
@@ -2415,19 +2420,6 @@ int64_t pair_slots() {
     return cache = -1;
   }
   return cache = static_cast<int64_t>(clusters) * 2;
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  if (fn == nullptr) {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
-  }
-  return fn;
 }
 
 // Row-major FP32 matrix [rows x cols] (cols innermost) with boxes of

@@ -3,9 +3,14 @@
 // and bounded waits that give up instead of hanging.
 #pragma once
 #include <cuda.h>
+#include <cudaTypedefs.h>
 #include <stdint.h>
 
 namespace sk {
+
+// cuTensorMapEncodeTiled of the driver, or null (sk_tc.cu).
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
+
 namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -105,6 +110,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const A
         return false;
       }
     }
+  }
+}
+
+// Bounded wait that ignores the abort flag (used only to drain in-flight
+// asynchronous work on the way out).
+__device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+  const uint64_t t0 = globaltimer();
+  while (!mbar_try_wait(bar, parity)) {
+    if (globaltimer() - t0 > limit_ns) return;
   }
 }
 

@@ -1,0 +1,669 @@
+// sk_tc32.cu -- FP32 form of the left sketch Y[k x n] = S[k x m] A[m x n] on
+// the tensor cores (tcgen05 + TMEM), every FP32 operand as the exact sum of
+// three BF16 values.
+//
+// The local multiply of the paper's Alg. 1 with the random operand
+// regenerated tile by tile, as k_sketch_fp32_simt does it on the CUDA cores.
+// Those are what bounded that kernel: it reached half of their 80 TFLOP/s,
+// and its 128 x 256 tiles cover a 333-column A to 65 %.  A 24-bit significand
+// splits without error into three of 8 bits, x = x1 + x2 + x3 (round to
+// nearest each time), and of the nine products of two such sums six carry
+// everything above 2^-24 of the whole:
+//   main   s1 a1
+//   cross  s1 a2 + s2 a1 + s2 a2 + s1 a3 + s3 a1
+// each exact in the tensor core, summed in FP32.  The tensor core truncates
+// where an FMA rounds, which shrinks a sum by about 2^-26 per K step, so the
+// two groups have accumulators of their own (the cross terms are 2^-8 of the
+// main ones, and so is what they lose) and the main one is a chain of at most
+// 6 or 8 stages that is added, with IEEE adds, to the ones before it.  A
+// Rademacher S is exact in one BF16 value: s1 a1, then s1 a2 + s1 a3.
+//
+// A CTA owns a 128 x NT tile of Y (NT <= 256: two accumulators of NT TMEM
+// columns) and a list of (tile, split of m) items:
+//   warp 0       TMEM allocation, MMA issuer: per stage of 32 rows of m
+//                2 K steps x 6 (3) tcgen05.mma kind::f16, M = 128, N = NT;
+//   warps 1-4    epilogue: a finished chain leaves TMEM (the item's last one
+//                with the cross sums) through staging tiles and the TMA for
+//                the item's FP32 partial (store, later chains add);
+//   warps 5-20   workers, two groups of 8 that take turns on stages: load the
+//                stage's rows of A (any alignment), generate the S tile while
+//                they arrive, split both into their operand layouts.
+// The workers bound it: 4096 generated entries and 32 NT split elements per
+// stage keep the issue slots 50 % busy, the MMAs the tensor pipe 21 %.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <string.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "sk_internal.h"
+#include "sk_rng.cuh"
+#include "sk_tc.cuh"
+
+namespace sk {
+namespace {
+
+using namespace tc;
+
+constexpr int BM = 128;      // rows of S per tile
+constexpr int SL = 32;       // rows of m per stage
+constexpr int SLOTS = 3;     // stages in the ring
+constexpr int NCH = 4;       // most 64-column chunks of a tile
+// Most stages per chain of the main accumulator: 192 rows of m (Rademacher
+// products are BF16 values and truncate less: 1024).
+constexpr int CHAIN = 6, CHAIN_LONG = 8, CHAIN_R = 32;
+constexpr int64_t kLongRows = 16384;  // rows of m from which chains are CHAIN_LONG
+constexpr int N_EPI = 4;
+constexpr int GROUPS = 2, GROUP_WARPS = 8;
+constexpr int W_EPI0 = 1, W_WORK0 = W_EPI0 + N_EPI;
+constexpr int THREADS = 32 * (W_WORK0 + GROUPS * GROUP_WARPS);
+
+// Slot of a stage: the parts of S (K-major core matrices without swizzle, two
+// slabs of 16 columns each), then those of A (MN-major with the 128-byte
+// swizzle: chunks of 64 columns x 32 rows).
+constexpr uint32_t S_SLAB = BM * 16 * 2;        // 4096
+constexpr uint32_t S_PART = 2 * S_SLAB;         // 8192
+constexpr uint32_t A_CHUNK = SL * 64 * 2;       // 4096
+constexpr uint32_t OFF_A = 3 * S_PART;
+constexpr uint32_t SLOT_MAX = OFF_A + 3 * NCH * A_CHUNK;
+// Staging tile of a drain: 32 rows x 16 columns with the 64-byte swizzle
+// (4-column unit u of row r at u ^ (r / 2 mod 4)).  Behind the ring an
+// epilogue warp has one, or four where tiles of fewer columns leave room.
+constexpr uint32_t EPI_TILE = 32 * 16 * 4;
+constexpr uint32_t OFF_BAR = SLOTS * SLOT_MAX + N_EPI * EPI_TILE;
+constexpr uint32_t NUM_BARS = 2 * SLOTS + 3;
+constexpr uint32_t OFF_MISC = OFF_BAR + NUM_BARS * 8;  // abort flag, TMEM slot, chain flags
+constexpr uint32_t SMEM = OFF_MISC + 16 + 4 * 4 + 1024;  // + slack for 1 KB alignment
+static_assert(SMEM <= 227 * 1024, "shared memory budget");
+static_assert(SLOT_MAX % 1024 == 0 && OFF_A % 1024 == 0, "swizzle atoms on 1 KB boundaries");
+static_assert(SLOTS * (SLOT_MAX - 3 * A_CHUNK) + N_EPI * 4 * EPI_TILE <= OFF_BAR, "staging tiles");
+static_assert(GROUPS <= SLOTS, "worker groups vs ring depth");
+
+// |a| above this rounds to an infinite BF16; such a value is truncated.
+constexpr float kRoundsToInf = 0x1.fep127f;
+// Magnitudes from 2^-110 on split without error; an item's tile of A whose
+// largest magnitude is below this is multiplied in FP32 FMAs instead.
+constexpr float kTiny = 0x1p-100f;
+// What the workers saw in an item's rows of A.
+constexpr int kSawTiny = 1, kSawNormal = 2;
+
+struct F32Params {
+  const float* A;
+  int64_t lda;
+  float* part;  // partials [splits][P][ldp]
+  int64_t P, Q, L, ldp;
+  int64_t chunk;  // contracted length per split (a multiple of SL)
+  int tiles_p, tiles_q, nitems;
+  int nt;     // columns per tile, a multiple of 64
+  int chain;  // stages per accumulation chain
+  int vec2;   // rows of A on 8-byte boundaries
+  int dist;
+  PhiloxRoundKeys rk;
+  int* status;
+  uint64_t timeout_ns;
+};
+
+struct Item {
+  int64_t p0, q0, lbeg, lend;
+  int z, nsteps, nchains;
+};
+
+__device__ __forceinline__ Item get_item(const F32Params& p, int idx) {
+  Item it;
+  const int t = idx / p.tiles_p;
+  it.p0 = static_cast<int64_t>(idx - t * p.tiles_p) * BM;
+  it.q0 = static_cast<int64_t>(t % p.tiles_q) * p.nt;
+  it.z = t / p.tiles_q;
+  it.lbeg = static_cast<int64_t>(it.z) * p.chunk;
+  it.lend = min(p.L, it.lbeg + p.chunk);
+  it.nsteps = static_cast<int>((it.lend - it.lbeg + SL - 1) / SL);
+  it.nchains = (it.nsteps + p.chain - 1) / p.chain;
+  return it;
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo_elem, float hi_elem) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo_elem, hi_elem);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ float2 unpack_bf16(uint32_t w) {
+  return f2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+// x minus the BF16 values packed in w (exact: both have at most 24 bits and
+// the difference fits)
+__device__ __forceinline__ float2 minus_bf16(float2 x, uint32_t w) {
+  return __ffma2_rn(unpack_bf16(w), f2(-1.0f, -1.0f), x);
+}
+
+// The two elements of x as sums of three BF16 values, packed by part.
+// HUGE_OK: elements that would round to infinity are truncated.
+template <bool HUGE_OK>
+__device__ __forceinline__ void split3(float2 x, uint32_t (&w)[3]) {
+  w[0] = pack_bf16(x.x, x.y);
+  if (HUGE_OK) {
+    if (fabsf(x.x) >= kRoundsToInf && !isinf(x.x))
+      w[0] = (w[0] & 0xffff0000u) | (__float_as_uint(x.x) >> 16);
+    if (fabsf(x.y) >= kRoundsToInf && !isinf(x.y))
+      w[0] = (w[0] & 0x0000ffffu) | (__float_as_uint(x.y) & 0xffff0000u);
+  }
+  const float2 r = minus_bf16(x, w[0]);
+  w[1] = pack_bf16(r.x, r.y);
+  const float2 q = minus_bf16(r, w[1]);
+  w[2] = pack_bf16(q.x, q.y);
+}
+
+// A row of an item's tile in FP32 FMAs, for a tile of A too small in
+// magnitude to split (rare: all of it below 2^-100).
+__device__ __noinline__ void slow_item(const F32Params& p, int64_t row, int64_t q0, int64_t q1,
+                                       int64_t l0, int64_t l1, float* out) {
+  const PhiloxKey key{p.rk.k[0], p.rk.k[1]};
+  for (int64_t c = q0; c < q1; c += 8) {
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const int nc = static_cast<int>(min(static_cast<int64_t>(8), q1 - c));
+    for (int64_t l = l0; l < l1; l += 4) {
+      const float4 g = gen4(p.dist, key, static_cast<uint32_t>(row), static_cast<uint32_t>(l));
+      const float gg[4] = {g.x, g.y, g.z, g.w};
+      for (int i = 0; i < 4 && l + i < l1; ++i) {
+        const float* a = p.A + (l + i) * p.lda + c;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (j < nc) acc[j] = __fmaf_rn(gg[i], a[j], acc[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (j < nc) out[c + j] = acc[j];
+  }
+}
+
+template <int DIST>
+__global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_constant__ CUtensorMap pmap, const F32Params p) {
+  constexpr int NS = DIST == kRademacher ? 1 : 3;  // parts of S
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t bar0 = sbase + OFF_BAR;
+  // full: a worker group has written the slot; empty: its MMAs have completed
+  auto full = [&](int i) { return bar0 + 8u * i; };
+  auto empty = [&](int i) { return bar0 + 8u * (SLOTS + i); };
+  const uint32_t acc_full = bar0 + 8u * (2 * SLOTS);
+  const uint32_t acc_empty = acc_full + 8u;
+  const uint32_t drain_bar = acc_full + 16u;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_MISC);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_MISC + 4);
+  // kSawTiny / kSawNormal of the last four items: the workers are at most
+  // three stages, hence three items, ahead of the epilogue
+  int* saw = reinterpret_cast<int*>(smem + OFF_MISC + 16);
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < SLOTS; ++i) {
+      mbar_init(full(i), GROUP_WARPS);
+      mbar_init(empty(i), 1);
+    }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, N_EPI);
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    for (int i = 0; i < 4; ++i) saw[i] = 0;
+    mbar_fence_init();
+  }
+  if (warp == 0) {
+    tmem_alloc(smem_u32(tmem_slot), 512u);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_wait();
+  pdl_trigger();
+  const uint32_t tmem = *tmem_slot;
+  const Abort ab{abort_flag, p.status, p.timeout_ns};
+  const uint32_t a_part = static_cast<uint32_t>(p.nt / 64) * A_CHUNK;  // one part of A in a slot
+  const uint32_t slot_bytes = OFF_A + 3u * a_part;
+  const int first_item = static_cast<int>(blockIdx.x), item_step = static_cast<int>(gridDim.x);
+
+  if (warp == 0) {
+    if (lane == 0) {
+      const uint32_t idesc =
+          idesc_bf16_f32(BM, static_cast<uint32_t>(p.nt)) | (1u << 16);  // B is MN-major
+      const uint64_t a_base = smem_desc(sbase, 128u, 256u);
+      const uint64_t b_base = smem_desc_sw128(sbase + OFF_A, A_CHUNK, 1024u);
+      int g = 0, gc = 0, j = 0;
+      bool stop = false;
+      for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+        const int nsteps = get_item(p, idx).nsteps;
+        int in_chain = 0;
+        for (int s = 0; s < nsteps; ++s, ++g) {
+          const int so = g % SLOTS;
+          if (in_chain == 0 && gc > 0) {
+            // every epilogue warp has read the last chain (and its item's flags)
+            if (!mbar_wait(acc_empty, (gc - 1) & 1, ab, 0x25, gc)) {
+              stop = true;
+              break;
+            }
+            if (s == 0) saw[(j - 1) & 3] = 0;
+          }
+          if (!mbar_wait(full(so), (g / SLOTS) & 1, ab, 0x22, g)) {
+            stop = true;
+            break;
+          }
+          tc_fence_after();
+          // offsets are multiples of 16 B below 256 KB: added to the low word
+          const uint64_t a0 = a_base + ((static_cast<uint32_t>(so) * slot_bytes) >> 4);
+          const uint64_t b0 = b_base + ((static_cast<uint32_t>(so) * slot_bytes) >> 4);
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            auto mma = [&](int sp, int ap, uint32_t col, uint32_t acc) {
+              mma_bf16(tmem + col, a0 + ((sp * S_PART + ks * S_SLAB) >> 4),
+                       b0 + ((static_cast<uint32_t>(ap) * a_part + ks * 2048u) >> 4), idesc, acc);
+            };
+            mma(0, 0, 0u, in_chain > 0 || ks > 0 ? 1u : 0u);
+            mma(0, 1, 256u, s > 0 || ks > 0 ? 1u : 0u);
+            mma(0, 2, 256u, 1u);
+            if (NS == 3) {
+              mma(1, 0, 256u, 1u);
+              mma(1, 1, 256u, 1u);
+              mma(2, 0, 256u, 1u);
+            }
+          }
+          mma_commit(empty(so));
+          if (++in_chain == p.chain || s == nsteps - 1) {
+            mma_commit(acc_full);
+            in_chain = 0;
+            ++gc;
+          }
+        }
+      }
+      mma_commit(drain_bar);
+      drain_wait(drain_bar, 0, 200000000ull);
+    }
+  } else if (warp < W_WORK0) {
+    // ---- epilogue: lanes are accumulator rows, main in columns 0 .. nt - 1,
+    // cross in 256 .. ----
+    const int quarter = warp & 3;
+    const int ntile = p.nt == 64 * NCH ? 1 : 4;
+    uint8_t* tiles = smem + SLOTS * slot_bytes + (warp - W_EPI0) * ntile * EPI_TILE;
+    const uint32_t usw = (static_cast<uint32_t>(lane) >> 1) & 3u;
+    int gc = 0, j = 0;
+    bool stop = false;
+    for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+      const Item it = get_item(p, idx);
+      float* part = p.part + static_cast<int64_t>(it.z) * p.P * p.ldp;
+      const int64_t r0 = it.p0 + quarter * 32;
+      for (int c0 = 0; c0 < it.nchains; ++c0, ++gc) {
+        const bool ok = mbar_wait(acc_full, gc & 1, ab, 0x34, gc);
+        if (!__all_sync(0xffffffffu, ok)) {
+          stop = true;
+          break;
+        }
+        tc_fence_after();
+        const bool first = c0 == 0, last = c0 == it.nchains - 1;
+        // the earlier chains' adds have been performed: those of one element
+        // stay in chain order
+        if (lane == 0) bulk_wait<0>();
+        __syncwarp();
+        const bool slow = last && *static_cast<volatile int*>(saw + (j & 3)) == kSawTiny;
+        const int nchunk = r0 >= p.P || slow
+                               ? 0
+                               : static_cast<int>((min(static_cast<int64_t>(p.nt), p.Q - it.q0) + 31) / 32);
+        if (slow && r0 + lane < p.P)
+          slow_item(p, r0 + lane, it.q0, min(p.Q, it.q0 + p.nt), it.lbeg, it.lend,
+                    part + (r0 + lane) * p.ldp);
+        int nb = 0;
+        for (int ci = 0; ci < nchunk; ++ci) {
+          uint32_t v[32], w[32];
+          const uint32_t src =
+              tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(ci * 32);
+          tmem_ld32(src, v);
+          if (last) {
+            tmem_ld32(src + 256u, w);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              // the cross terms of an infinite or NaN element mean nothing:
+              // the main sum is infinite or NaN already
+              const float c = __uint_as_float(w[i]);
+              if (fabsf(c) <= 0x1.fffffep127f)
+                v[i] = __float_as_uint(__fadd_rn(__uint_as_float(v[i]), c));
+            }
+          } else {
+            tmem_ld_wait();
+          }
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const int64_t col = it.q0 + ci * 32 + 16 * half;
+            if (col >= p.Q) break;
+            if (nb >= ntile) {  // the TMA has read what the tile held before
+              if (lane == 0) {
+                if (ntile == 1)
+                  bulk_wait_read<0>();
+                else
+                  bulk_wait_read<3>();
+              }
+              __syncwarp();
+            }
+            uint8_t* tile = tiles + (nb % ntile) * EPI_TILE;
+            ++nb;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              *reinterpret_cast<float4*>(tile + lane * 64 + ((static_cast<uint32_t>(q) ^ usw) << 4)) =
+                  make_float4(__uint_as_float(v[16 * half + 4 * q]),
+                              __uint_as_float(v[16 * half + 4 * q + 1]),
+                              __uint_as_float(v[16 * half + 4 * q + 2]),
+                              __uint_as_float(v[16 * half + 4 * q + 3]));
+            fence_proxy_async_smem();  // the tile is read by the TMA
+            __syncwarp();
+            if (lane == 0) {
+              if (first)
+                tma_store_3d(&pmap, smem_u32(tile), static_cast<int32_t>(col),
+                             static_cast<int32_t>(r0), it.z);
+              else
+                tma_reduce_add_3d(&pmap, smem_u32(tile), static_cast<int32_t>(col),
+                                  static_cast<int32_t>(r0), it.z);
+              bulk_commit();
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty);
+      }
+    }
+    if (lane == 0) bulk_wait<0>();  // the last copies have completed
+  } else {
+    // ---- workers ----
+    const int grp = (warp - W_WORK0) / GROUP_WARPS;
+    const int w = (warp - W_WORK0) % GROUP_WARPS;
+    // Gaussian and uniform tasks: quad qd of row rbase + 64 i in both slabs
+    // (the lanes of a store phase write every bank once)
+    const uint32_t qd = static_cast<uint32_t>(lane) >> 3;
+    const uint32_t rbase = static_cast<uint32_t>(w * 8 + (lane & 7));
+    const uint32_t s_off =
+        (rbase & 7u) * 16u + (rbase >> 3) * 256u + (qd >> 1) * 128u + (qd & 1u) * 8u;
+    int g = 0, j = 0;
+    bool stop = false;
+    for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+      const Item it = get_item(p, idx);
+      const int g_item = g;
+      // columns of the tile: nfull whole chunks, then perhaps part of one,
+      // where lanes past the last column read that one again (what they
+      // contribute to is never read out)
+      const int ncols = static_cast<int>(min(static_cast<int64_t>(p.nt), p.Q - it.q0));
+      const int nfull = ncols / 64, nconv = (ncols + 63) / 64;
+      const int edge0 = min(64 * nfull + 2 * lane, ncols - 1);
+      const int edge1 = min(64 * nfull + 2 * lane + 1, ncols - 1);
+      for (int s = (grp + GROUPS - g_item % GROUPS) % GROUPS; s < it.nsteps; s += GROUPS) {
+        g = g_item + s;
+        const int so = g % SLOTS;
+        uint8_t* slot = smem + static_cast<uint32_t>(so) * slot_bytes;
+        const int64_t cbase = it.lbeg + static_cast<int64_t>(s) * SL;
+        bool ok = true;
+        float amax = 0.0f;
+        float hmax = 0.0f;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          // this warp's rows 16 half + 2 w, + 1 of the stage, columns 2 lane,
+          // + 1 of each chunk, in flight while the S rows are generated
+          float2 x[2][NCH];
+#pragma unroll
+          for (int j2 = 0; j2 < 2; ++j2) {
+            const int64_t l = cbase + 16 * half + 2 * w + j2;
+            const float* row = p.A + l * p.lda + it.q0;
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+              x[j2][c] = f2(0.0f, 0.0f);
+              if (l >= it.lend) continue;
+              if (c < nfull) {
+                const float* src = row + 2 * lane + 64 * c;
+                if (p.vec2)
+                  x[j2][c] = __ldg(reinterpret_cast<const float2*>(src));
+                else
+                  x[j2][c] = f2(__ldg(src), __ldg(src + 1));
+              } else if (c < nconv) {
+                x[j2][c] = f2(__ldg(row + edge0), __ldg(row + edge1));
+              }
+            }
+          }
+          if (half == 0) {  // the MMAs that read the slot last time have completed
+            ok = g < SLOTS || mbar_wait(empty(so), ((g / SLOTS) & 1) ^ 1, ab, 0x43, g);
+            if (!__all_sync(0xffffffffu, ok)) break;
+          }
+          // S rows 64 half .. 64 half + 63 (those past P are never read out)
+          if constexpr (DIST == kRademacher) {
+            const int r = 64 * half + (w & 1) * 32 + lane;  // and 8 columns per warp pair
+            if (it.p0 + r < p.P) {
+              const int kc = w >> 1;
+              const uint32_t c = static_cast<uint32_t>(cbase);
+              const uint4 x4 = rademacher_bits(p.rk, static_cast<uint32_t>(it.p0 + r), c >> 7);
+              const uint32_t ws = (c >> 5) & 3u;
+              const uint32_t b = (ws == 0 ? x4.x : ws == 1 ? x4.y : ws == 2 ? x4.z : x4.w) >> (8 * kc);
+              uint4 v;
+              v.x = 0x3F803F80u | ((b & 1u) << 15) | ((b & 2u) << 30);
+              v.y = 0x3F803F80u | ((b & 4u) << 13) | ((b & 8u) << 28);
+              v.z = 0x3F803F80u | ((b & 16u) << 11) | ((b & 32u) << 26);
+              v.w = 0x3F803F80u | ((b & 64u) << 9) | ((b & 128u) << 24);
+              *reinterpret_cast<uint4*>(slot + (kc >> 1) * S_SLAB + (r & 7) * 16 + (r >> 3) * 256 +
+                                        (kc & 1) * 128) = v;
+            }
+          } else {
+            const int64_t grow = it.p0 + rbase + 64 * half;
+            if (grow < p.P) {
+              const PhiloxRow pr = philox_row(p.rk, static_cast<uint32_t>(grow));
+              const uint32_t j0 = static_cast<uint32_t>(cbase >> 2) + qd;
+#pragma unroll
+              for (int slab = 0; slab < 2; ++slab) {
+                const float4 v = entries4<DIST>(pr, philox_col(p.rk, j0 + 4u * slab), p.rk);
+                uint32_t lo[3], hi[3];
+                split3<false>(f2(v.x, v.y), lo);
+                split3<false>(f2(v.z, v.w), hi);
+#pragma unroll
+                for (int pt = 0; pt < 3; ++pt)
+                  *reinterpret_cast<uint2*>(slot + pt * S_PART + slab * S_SLAB + half * 2048 +
+                                            s_off) = make_uint2(lo[pt], hi[pt]);
+              }
+            }
+          }
+          hmax = 0.0f;
+#pragma unroll
+          for (int j2 = 0; j2 < 2; ++j2)
+#pragma unroll
+            for (int c = 0; c < NCH; ++c)
+              hmax = fmaxf(hmax, fmaxf(fabsf(x[j2][c].x), fabsf(x[j2][c].y)));
+          amax = fmaxf(amax, hmax);
+          auto store = [&](auto huge) {
+#pragma unroll
+            for (int j2 = 0; j2 < 2; ++j2) {
+              const int r = 16 * half + 2 * w + j2;
+              uint8_t* dst =
+                  slot + OFF_A + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + ((lane & 3) << 2);
+#pragma unroll
+              for (int c = 0; c < NCH; ++c) {
+                if (c >= nconv) break;
+                uint32_t q[3];
+                split3<decltype(huge)::value>(x[j2][c], q);
+#pragma unroll
+                for (int pt = 0; pt < 3; ++pt)
+                  *reinterpret_cast<uint32_t*>(dst + pt * a_part + c * A_CHUNK) = q[pt];
+              }
+            }
+          };
+          if (hmax >= kRoundsToInf)
+            store(std::true_type{});
+          else
+            store(std::false_type{});
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
+          stop = true;
+          break;
+        }
+        const bool normal = __any_sync(0xffffffffu, amax >= kTiny);
+        const bool tiny = __any_sync(0xffffffffu, amax > 0.0f);
+        fence_proxy_async_smem();  // the slot is read by the tensor core
+        __syncwarp();
+        if (lane == 0) {
+          if (tiny) atomicOr(saw + (j & 3), normal ? kSawNormal : kSawTiny);
+          mbar_arrive(full(so));
+        }
+      }
+      g = g_item + it.nsteps;
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    __syncwarp();
+    tmem_dealloc(tmem, 512u);
+  }
+}
+
+// ---- host side ----
+int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms <= 0) sms = 148;
+  }
+  return sms;
+}
+
+struct F32Plan {
+  int nt, splits, chain;
+  int64_t tiles_p, tiles_q, chunk, ldp;
+};
+
+F32Plan plan_f32(const GemmShape& s, int dist = kGaussian) {
+  F32Plan pl;
+  const int64_t chunks = (s.Q + 63) / 64;
+  pl.tiles_q = (chunks + NCH - 1) / NCH;
+  pl.nt = static_cast<int>((chunks + pl.tiles_q - 1) / pl.tiles_q) * 64;
+  pl.tiles_p = (s.P + BM - 1) / BM;
+  pl.ldp = (s.Q + 3) / 4 * 4;
+  // splits of m that fill whole waves of CTAs, each at least one stage per
+  // worker group
+  const int64_t tiles = pl.tiles_p * pl.tiles_q, sms = sm_count();
+  const int64_t steps = (s.L + SL - 1) / SL;
+  const int64_t smax = std::max<int64_t>(1, std::min<int64_t>(steps / GROUPS, 64));
+  int64_t best = 1;
+  double best_fill = -1.0;
+  for (int64_t sp = 1; sp <= smax; ++sp) {
+    const int64_t items = tiles * sp, waves = (items + sms - 1) / sms;
+    const double fill = static_cast<double>(items) / static_cast<double>(waves * sms);
+    if (fill > best_fill + 0.02) {
+      best_fill = fill;
+      best = sp;
+    }
+    if (items >= 4 * sms) break;
+  }
+  int64_t per = (steps + best - 1) / best;
+  pl.chunk = per * SL;
+  pl.splits = static_cast<int>((steps + per - 1) / per);
+  const int64_t cap = dist == kRademacher ? CHAIN_R : s.L >= kLongRows ? CHAIN_LONG : CHAIN;
+  const int64_t nchains = (per + cap - 1) / cap;
+  pl.chain = static_cast<int>((per + nchains - 1) / nchains);
+  return pl;
+}
+
+// The partials [splits][P][ldp] in boxes of 16 columns x 32 rows with the
+// 64-byte swizzle.
+bool encode_partials(CUtensorMap* map, float* part, int64_t Q, int64_t P, int splits, int64_t ldp) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+  if (enc == nullptr) return false;
+  const cuuint64_t gdim[3] = {static_cast<cuuint64_t>(Q), static_cast<cuuint64_t>(P),
+                              static_cast<cuuint64_t>(splits)};
+  const cuuint64_t gstride[2] = {static_cast<cuuint64_t>(ldp) * 4,
+                                 static_cast<cuuint64_t>(P) * static_cast<cuuint64_t>(ldp) * 4};
+  const cuuint32_t box[3] = {16, 32, 1}, estride[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, part, gdim, gstride, box, estride,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int DIST>
+cudaError_t launch_f32(const CUtensorMap& pmap, const F32Params& p, unsigned grid,
+                       cudaStream_t st) {
+  static bool done = false;
+  if (!done) {
+    const cudaError_t e = cudaFuncSetAttribute(k_sketch_fp32_left<DIST>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    if (e != cudaSuccess) return e;
+    done = true;
+  }
+  return launch_overlapped(k_sketch_fp32_left<DIST>, dim3(grid), dim3(THREADS), SMEM, st, 1, pmap,
+                           p);
+}
+
+}  // namespace
+
+// The left sketch with at least two stages of m.  Time, and relative
+// Frobenius error against 64 bits, with FP32 FMAs on the CUDA cores and here
+// (Gaussian S; m x n, k):
+//   4096 x 256, 64       39 -> 18 us      2.3e-7 -> 1.5e-7
+//   30011 x 333, 666     644 -> 207 us    5.4e-7 -> 2.5e-7
+//   65536 x 512, 1024    1590 -> 647 us   1.1e-6 -> 2.6e-7
+//   16384 x 100, 300     85 -> 36 us      3.2e-7 -> 2.1e-7
+//   200000 x 16, 16      754 -> 126 us    1.1e-6 -> 2.3e-7
+//   1000 x 1, 1          44 -> 17 us      1.3e-7 -> 2.3e-8
+//   64 x 32, 64          21 -> 16 us      1.5e-7 -> 6.7e-8
+//   32 x 512, 512        15.2 -> 17.5 us  (one stage: stays on the CUDA cores)
+// Chains of 11, 19 and 32 stages had errors of 3.4e-7, 5.8e-7 and 8.3e-7.
+bool tc32_applies(const GemmShape& s) {
+  if (!s.left || s.L < 2 * SL) return false;
+  const F32Plan pl = plan_f32(s);
+  // (a k of more than 65535 tiles is refused, as the CUDA-core form does)
+  if (s.P > 65535LL * (s.Q > 128 ? 128 : 256)) return false;
+  // 32-bit item numbers, and strides that a tensor map holds
+  return pl.tiles_p * pl.tiles_q * pl.splits < (int64_t(1) << 31) && s.Q < (int64_t(1) << 31) &&
+         s.P * pl.ldp * 4 < (int64_t(1) << 40);
+}
+
+size_t tc32_workspace_bytes(const GemmShape& s) {
+  const F32Plan pl = plan_f32(s);
+  return static_cast<size_t>(pl.splits) * s.P * pl.ldp * sizeof(float);
+}
+
+cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
+                             float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st) {
+  if (ws == nullptr || ws_bytes < tc32_workspace_bytes(s)) return cudaErrorInvalidValue;
+  const F32Plan pl = plan_f32(s, h->dist);
+  F32Params p;
+  memset(&p, 0, sizeof(p));
+  p.A = A;
+  p.lda = lda;
+  p.part = static_cast<float*>(ws);
+  p.P = s.P;
+  p.Q = s.Q;
+  p.L = s.L;
+  p.ldp = pl.ldp;
+  p.chunk = pl.chunk;
+  p.tiles_p = static_cast<int>(pl.tiles_p);
+  p.tiles_q = static_cast<int>(pl.tiles_q);
+  p.nitems = static_cast<int>(pl.tiles_p * pl.tiles_q * pl.splits);
+  p.nt = pl.nt;
+  p.chain = pl.chain;
+  p.vec2 = reinterpret_cast<uintptr_t>(A) % 8 == 0 && lda % 2 == 0;
+  p.dist = h->dist;
+  p.rk = round_keys(make_key(h->seed));
+  p.status = h->d_status;
+  p.timeout_ns = h->wait_limit_ns;
+  CUtensorMap pmap;
+  if (!encode_partials(&pmap, p.part, s.Q, s.P, pl.splits, pl.ldp)) return cudaErrorInvalidValue;
+  const unsigned grid = static_cast<unsigned>(std::min(p.nitems, sm_count()));
+  prof_mark(h->prof_start, st);
+  const cudaError_t e = h->dist == kRademacher ? launch_f32<kRademacher>(pmap, p, grid, st)
+                        : h->dist == kUniform  ? launch_f32<kUniform>(pmap, p, grid, st)
+                                               : launch_f32<kGaussian>(pmap, p, grid, st);
+  prof_mark(h->prof_stop, st);
+  if (e != cudaSuccess) return e;
+  count_launches(1);
+  return splitk_reduce(p.part, pl.splits, s.P, s.Q, pl.ldp, h->scale, Y, ldy, st);
+}
+
+}  // namespace sk
