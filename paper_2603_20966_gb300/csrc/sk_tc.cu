@@ -683,10 +683,14 @@ __device__ __noinline__ bool drain_chain_left(uint32_t tmem, int quarter, int co
 // Whether a launch runs the separate ring of S tiles (Cfg::SRING): the
 // wide pair kernels that generate Gaussian or uniform S.  Rademacher tiles
 // cost the workers little and their workers split A, so one ring of both
-// operands serves them; a stored S arrives with the A tile.
-template <int DIST, bool PAIR, bool NARROW>
-using LeftCfg =
-    Cfg<PAIR, NARROW, PAIR && !NARROW && (DIST == kGaussian || DIST == kUniform || DIST == kMixed)>;
+// operands serves them; a stored S arrives with the A tile.  Batches only
+// where the epilogue warps certify A: a server's batches, whose A is split
+// before the launch, took 4.44 ms against 4.34 ms for a burst of 48 with the
+// odd CTA's relay in their many short items.
+template <int DIST, bool PAIR, bool NARROW, bool EC>
+using LeftCfg = Cfg<PAIR, NARROW,
+                    PAIR && !NARROW && (DIST == kGaussian || DIST == kUniform ||
+                                        (DIST == kMixed && EC))>;
 
 // Persistent left-sketch kernel: each pair (or single CTA) runs its list of
 // items back to back; ring positions, barrier phases and accumulation chains
@@ -699,7 +703,7 @@ template <int DIST, bool PAIR, bool NARROW = false, bool EC = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_sketch_bf16x2_left(const __grid_constant__ LeftSched sc,
                          const __grid_constant__ LeftProblem one) {
-  using C = LeftCfg<DIST, PAIR, NARROW>;
+  using C = LeftCfg<DIST, PAIR, NARROW, EC>;
   constexpr bool SRING = C::NSS > C::NSO;
   // the odd CTA's second warp passes its landed A tiles on to the MMA issuer
   constexpr bool RELAY = SRING && !EC;
@@ -775,9 +779,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (PAIR) cluster_sync();  // the peer's barriers exist before any remote arrive
   tc_fence_after();
   // what this launch reads and overwrites is ready once the one before it
-  // has finished; the reduction may set itself up beside this kernel
+  // has finished; a single sketch's reduction may set itself up beside this
+  // kernel (a batch's would wait for milliseconds on the registers that a
+  // server's kernels for the next requests run on)
   pdl_wait();
-  pdl_trigger();
+  if (DIST != kMixed) pdl_trigger();
   const uint32_t tmem = *tmem_slot;
   const Abort ab{abort_flag, sc.status, sc.timeout_ns};
   // barriers of the even CTA, addressed from either CTA
@@ -2379,7 +2385,7 @@ cudaError_t set_smem_attr() {
   if (done) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       LeftCfg<DIST, PAIR, NARROW>::SMEM);
+                                       LeftCfg<DIST, PAIR, NARROW, EC>::SMEM);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -2411,7 +2417,7 @@ int64_t pair_slots() {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_config<true>(&cfg, attr, dim3(2, 1, 1), nullptr);
-  cfg.dynamicSmemBytes = LeftCfg<kMixed, true, false>::SMEM;
+  cfg.dynamicSmemBytes = LeftCfg<kMixed, true, false, false>::SMEM;
   int clusters = 0;
   if (cudaOccupancyMaxActiveClusters(&clusters, k_sketch_bf16x2_left<kMixed, true>, &cfg) !=
           cudaSuccess ||
@@ -2609,13 +2615,13 @@ cudaError_t launch_left(const LeftSched& sc, const LeftProblem& one, int64_t uni
   const dim3 grid(static_cast<unsigned>(units * (PAIR ? 2 : 1)), 1, 1);
   if (sc.claim == nullptr)
     return launch_overlapped(k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, grid, dim3(NTHREADS),
-                             LeftCfg<DIST, PAIR, NARROW>::SMEM, st, PAIR ? 2 : 1, sc, one);
+                             LeftCfg<DIST, PAIR, NARROW, EC>::SMEM, st, PAIR ? 2 : 1, sc, one);
   e = cudaMemsetAsync(sc.claim, 0, sizeof(int), st);  // the work list starts unclaimed
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_config<PAIR>(&cfg, attr, grid, st);
-  cfg.dynamicSmemBytes = LeftCfg<DIST, PAIR, NARROW>::SMEM;
+  cfg.dynamicSmemBytes = LeftCfg<DIST, PAIR, NARROW, EC>::SMEM;
   return cudaLaunchKernelEx(&cfg, k_sketch_bf16x2_left<DIST, PAIR, NARROW, EC>, sc, one);
 }
 
