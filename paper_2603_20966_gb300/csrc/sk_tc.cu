@@ -206,8 +206,18 @@ struct alignas(128) LeftProblem {
   CUtensorMap pmap;
 };
 
+// Rows of S that each CTA of a pair takes of a 256-row tile with `rem` rows
+// of S left: half of them, in whole 32-row boxes of the drain, so that both
+// CTAs generate the same share of a problem's last tile (the first CTA took
+// up to 128 of them before, while the second waited for it: batch of 256
+// 4.962 -> 4.859 ms, left 48611 x 301, k = 602 101 -> 99.6 us).
+__host__ __device__ inline int pair_rows(int64_t rem) {
+  return rem >= 2 * BM ? BM : static_cast<int>((rem + 63) / 64) * 32;
+}
+
 // A unit of work: tile (tp, tq) of split z of problem `prob`.  With pairs,
-// tp indexes 256-row tiles and the CTA of rank r takes rows 128 r .. of it.
+// tp indexes 256-row tiles and the CTA of rank r takes rows pair_rows r .. of
+// it.
 struct LeftItem {
   int prob, tp, tq, z;
 };
@@ -332,7 +342,7 @@ __global__ void __launch_bounds__(256)
 // Per-item geometry shared by every role.
 struct ItemGeo {
   const LeftProblem* pr;
-  int64_t P;      // rows of S (copied: the workers' loop keeps it in a register)
+  int64_t P;      // end of this CTA's rows of S (p0 its first; kept in a register)
   PhiloxKey key;  // (likewise)
   int64_t p0, q0, lbeg, lend;
   int nsteps, nt, nmma, nh, bh, cols, dist;
@@ -358,7 +368,6 @@ __device__ __forceinline__ ItemGeo item_geo(const LeftSched& sc, const LeftProbl
   const LeftItem it = left_item<DIST>(sc, idx);
   ItemGeo g;
   g.pr = DIST == kMixed ? sc.probs + it.prob : &one;
-  g.P = g.pr->P;
   g.key = g.pr->key;
   g.nt = g.pr->nt;
   g.dist = g.pr->dist;
@@ -366,7 +375,10 @@ __device__ __forceinline__ ItemGeo item_geo(const LeftSched& sc, const LeftProbl
   g.nh = g.nt > 256 ? 256 : g.nt;
   g.bh = PAIR ? g.nh / 2 : g.nh;
   g.cols = g.nmma * g.bh;
-  g.p0 = static_cast<int64_t>(it.tp) * (PAIR ? 2 * BM : BM) + static_cast<int64_t>(rank) * BM;
+  const int64_t t0 = static_cast<int64_t>(it.tp) * (PAIR ? 2 * BM : BM);
+  const int rows = PAIR ? pair_rows(g.pr->P - t0) : BM;
+  g.p0 = t0 + static_cast<int64_t>(rank) * rows;
+  g.P = min(g.pr->P, g.p0 + rows);
   g.q0 = static_cast<int64_t>(it.tq) * g.nt;
   g.lbeg = static_cast<int64_t>(it.z) * g.pr->chunk;
   g.lend = min(g.pr->L, g.lbeg + g.pr->chunk);
@@ -552,9 +564,10 @@ __device__ __noinline__ bool drain_chain_tma(uint32_t tmem, int quarter, int col
   if (!__all_sync(0xffffffffu, ok)) return false;  // tcgen05.ld below is warp-collective
   tc_fence_after();
   const int32_t y = static_cast<int32_t>(ig.p0 + quarter * 32);
+  const bool mine = ig.p0 + quarter * 32 < ig.P;  // rows past P are nobody's or the other CTA's
   const uint32_t sw = static_cast<uint32_t>(lane) & 7u;
   int nb = 0;
-  for (int ci = colset; ci * 32 < (ig.nmma - 1) * 256 + ig.nh; ci += 2, ++nb) {
+  for (int ci = colset; mine && ci * 32 < (ig.nmma - 1) * 256 + ig.nh; ci += 2, ++nb) {
     uint32_t v[32];
     tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(ci * 32),
               v);
@@ -615,7 +628,7 @@ __device__ __noinline__ bool drain_chain_left(uint32_t tmem, int quarter, int co
   const int lane = threadIdx.x & 31;
   const int rsub = lane >> 2;       // row within a group of 8 (read side)
   const int csub = (lane & 3) * 4;  // first of 4 columns (read side)
-  const int64_t P = ig.pr->P, Q = ig.pr->Q, ldp = ig.pr->ldp;
+  const int64_t P = ig.P, Q = ig.pr->Q, ldp = ig.pr->ldp;
   const bool vec_ok = (ldp % 4) == 0;
   const bool ok = mbar_wait(acc_full, gc & 1, ab, 0x34, gc);
   if (!__all_sync(0xffffffffu, ok)) return false;  // tcgen05.ld below is warp-collective
@@ -1061,8 +1074,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int idx = read_item_warp(j);
         if (idx < 0) break;
         const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
-        const int64_t P = ig.pr->P, Q = ig.pr->Q, ldp = ig.pr->ldp;
-        float* part_item = ig.pr->part + static_cast<int64_t>(ig.z) * P * ldp + ig.q0;
+        const int64_t P = ig.P, Q = ig.pr->Q, ldp = ig.pr->ldp;
+        float* part_item = ig.pr->part + static_cast<int64_t>(ig.z) * ig.pr->P * ldp + ig.q0;
         const bool vec_ok = (ldp % 4) == 0;
         const int nchains = (ig.nsteps + ig.coff + ig.chain - 1) / ig.chain;
         if (C::TDRAIN && ig.pr->tma_drain) {
@@ -2452,6 +2465,7 @@ struct LeftPlan {
   int splits;
   int64_t chunk;
   int64_t steps;             // stages of one item
+  int last_rows;             // rows of S per CTA of the last tile (of k)
 };
 
 // max_nt: the widest output tile (512 columns, two MMA instructions per K
@@ -2464,6 +2478,7 @@ LeftPlan left_geometry(const GemmShape& s, bool pair, int max_nt = NT_MAX) {
   pl.nt = s.Q > 256 && max_nt > 256 ? 512 : static_cast<int>(std::min<int64_t>((s.Q + gran - 1) / gran * gran, 256));
   pl.tiles_q = (s.Q + pl.nt - 1) / pl.nt;
   pl.tiles_p = (s.P + (pair ? 2 * BM : BM) - 1) / (pair ? 2 * BM : BM);
+  pl.last_rows = pair ? pair_rows(s.P - (pl.tiles_p - 1) * 2 * BM) : BM;
   pl.splits = 1;
   pl.chunk = (s.L + LK - 1) / LK * LK;
   pl.steps = pl.chunk / LK;
@@ -2552,8 +2567,8 @@ struct HostSched {
 // Items of every problem, longest (estimated) first; the kernel hands them
 // out in this order to whichever pair is free.  A stage costs about its
 // output columns plus a fixed 256 (generation, barriers), plus 640 for
-// Gaussian and uniform S (Box-Muller); launches use at most `max_units`
-// pairs (or CTAs).
+// Gaussian and uniform S (Box-Muller; less for a last tile of few rows);
+// launches use at most `max_units` pairs (or CTAs).
 void build_items(const std::vector<LeftPlan>& plans, const std::vector<int>& dists,
                  int64_t max_units, HostSched* hs) {
   struct Cand {
@@ -2564,13 +2579,15 @@ void build_items(const std::vector<LeftPlan>& plans, const std::vector<int>& dis
   for (size_t pi = 0; pi < plans.size(); ++pi) {
     const LeftPlan& pl = plans[pi];
     const double gen = dists[pi] == kRademacher ? 0.0 : 640.0;
-    const double cost = static_cast<double>(pl.steps) * (static_cast<double>(pl.nt) + 256.0 + gen);
+    const double mma = static_cast<double>(pl.nt) + 256.0;
+    const double cost = static_cast<double>(pl.steps) * (mma + gen);
+    const double last = static_cast<double>(pl.steps) * (mma + gen * pl.last_rows / BM);
     for (int64_t z = 0; z < pl.splits; ++z)
       for (int64_t tq = 0; tq < pl.tiles_q; ++tq)
         for (int64_t tp = 0; tp < pl.tiles_p; ++tp)
           cands.push_back({{static_cast<int>(pi), static_cast<int>(tp), static_cast<int>(tq),
                             static_cast<int>(z)},
-                           cost});
+                           tp == pl.tiles_p - 1 ? last : cost});
   }
   std::stable_sort(cands.begin(), cands.end(),
                    [](const Cand& a, const Cand& b) { return a.cost > b.cost; });
