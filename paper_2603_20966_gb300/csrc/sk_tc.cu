@@ -748,9 +748,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC + 4);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
-  const uint32_t rank = PAIR ? (cluster_ctarank() & 1u) : 0u;  // 0 = even (MMA issuer)
+  const uint32_t rank = PAIR ? uniform(cluster_ctarank() & 1u) : 0u;  // 0 = even (MMA issuer)
   const bool leader = rank == 0;
   // item queue: slot i holds the index of the item every role of the pair
   // (or single CTA) works on next; iq_full / iq_empty: written / read by all
@@ -797,7 +797,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // server's kernels for the next requests run on)
   pdl_wait();
   if (DIST != kMixed) pdl_trigger();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform(*tmem_slot);
   const Abort ab{abort_flag, sc.status, sc.timeout_ns};
   // barriers of the even CTA, addressed from either CTA
   const uint32_t lead_full_o = PAIR ? mapa_shared(full_o(0), 0u) : full_o(0);
@@ -894,11 +894,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
     }
   } else if (warp == WARP_MMA) {
-    if (lane == 0 && leader) {
+    if (leader) {  // the whole warp; one lane issues
+      const uint32_t el = elect_one();
       int g = 0, gc = 0;
       bool stop = false;
       for (int j = 0; !stop; ++j) {
-        const int idx = read_item(j);
+        const int idx = read_item_warp(j);
         if (idx < 0) break;
         const ItemGeo ig = item_geo<DIST, PAIR>(sc, one, idx, rank);
         const uint32_t idesc =
@@ -927,13 +928,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int ph = (s + ig.coff) & (ig.chain - 1);
           const bool chain_start = s == 0 || ph == 0;
           // a new chain may start only after every epilogue has read the last one
-          if (chain_start && gc > 0 && !mbar_wait(acc_empty, (gc - 1) & 1, ab, 0x25, gc)) {
+          if (chain_start && gc > 0 && !mbar_wait_warp(acc_empty, (gc - 1) & 1, ab, 0x25, gc)) {
             stop = true;
             break;
           }
-          if ((SRING && !mbar_wait(full_a(so), (g / C::NSO) & 1, ab, 0x22, g)) ||
-              (RELAY && !mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x22, g)) ||
-              !mbar_wait(full_o(ss), (g / C::NSS) & 1, ab, 0x22, g)) {
+          if ((SRING && !mbar_wait_warp(full_a(so), (g / C::NSO) & 1, ab, 0x22, g)) ||
+              (RELAY && !mbar_wait_warp(full_b(so), (g / C::NSO) & 1, ab, 0x22, g)) ||
+              !mbar_wait_warp(full_o(ss), (g / C::NSS) & 1, ab, 0x22, g)) {
             stop = true;
             break;
           }
@@ -953,27 +954,27 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                                        static_cast<uint32_t>(h) * hstride + ks * B_KSTEP) >> 4));
                 const uint32_t acc = (!chain_start || ks > 0 || pass > 0) ? 1u : 0u;
                 if (PAIR)
-                  mma_bf16_pair(tmem + static_cast<uint32_t>(h) * 256u, adesc, bdesc, idesc, acc);
+                  mma_bf16_pair(tmem + static_cast<uint32_t>(h) * 256u, adesc, bdesc, idesc, acc, el);
                 else
-                  mma_bf16(tmem + static_cast<uint32_t>(h) * 256u, adesc, bdesc, idesc, acc);
+                  mma_bf16(tmem + static_cast<uint32_t>(h) * 256u, adesc, bdesc, idesc, acc, el);
               }
             }
           }
           const bool chain_end = ph == ig.chain - 1 || s == ig.nsteps - 1;
           if (PAIR) {  // operands and accumulator are both CTAs'
-            mma_commit_pair_both(empty_o(ss));
-            if (chain_end) mma_commit_pair_both(acc_full);
+            mma_commit_pair_both(empty_o(ss), el);
+            if (chain_end) mma_commit_pair_both(acc_full, el);
           } else {
-            mma_commit(empty_o(ss));
-            if (chain_end) mma_commit(acc_full);
+            mma_commit(empty_o(ss), el);
+            if (chain_end) mma_commit(acc_full, el);
           }
           if (chain_end) ++gc;
         }
       }
       if (PAIR)
-        mma_commit_pair(drain_bar);
+        mma_commit_pair(drain_bar, el);
       else
-        mma_commit(drain_bar);
+        mma_commit(drain_bar, el);
       // every MMA has finished before this CTA reaches the closing barrier
       drain_wait(drain_bar, 0, 200000000ull);
     } else if (RELAY && lane == 0) {
@@ -1436,13 +1437,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC + 4);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   // a cluster holds two CTA pairs (cluster ranks 0-1 and 2-3) with the same
   // k rows and the same range of n on consecutive rows of m; the two CTAs of
   // equal rank in the two pairs hold the same rows of the S tile, and each
   // generates half of them and copies that half into its partner
-  const uint32_t cr = cluster_ctarank();
+  const uint32_t cr = uniform(cluster_ctarank());
   const uint32_t rank = cr & 1u;  // 0 = even CTA of the pair (MMA issuer)
   const uint32_t pairi = cr >> 1;
   const uint32_t lead_rank = cr & ~1u;          // the pair's even CTA
@@ -1507,7 +1508,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   cluster_sync();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform(*tmem_slot);
   const Abort ab{abort_flag, p.status, p.timeout_ns};
   const uint32_t lead_full_o = mapa_shared(full_o(0), lead_rank);
   const uint32_t partner_s_recv = mapa_shared(s_recv(0), partner);
@@ -1549,7 +1550,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
     }
   } else if (warp == WARP_MMA) {
-    if (lane == 0 && leader) {
+    if (leader) {  // the whole warp; one lane issues
+      const uint32_t el = elect_one();
       const uint32_t idesc = idesc_bf16_f32(256u, static_cast<uint32_t>(nq));
       // The single issuing thread's bookkeeping per stage bounds this kernel
       // (it issues 8 MMAs per 1024 tensor cycles), so the slot, phase and
@@ -1573,11 +1575,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const bool chain_start = in_chain == 0;
         // a chain starts once the epilogue has read the previous one
         if (chain_start && chain_no > 0 &&
-            !mbar_wait(acc_empty, (chain_no - 1) & 1, ab, 0x25, g)) {
+            !mbar_wait_warp(acc_empty, (chain_no - 1) & 1, ab, 0x25, g)) {
           stop = true;
           break;
         }
-        if (!mbar_wait(full_o(so), ph, ab, 0x22, g)) {
+        if (!mbar_wait_warp(full_o(so), ph, ab, 0x22, g)) {
           stop = true;
           break;
         }
@@ -1595,13 +1597,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               const uint64_t adesc =
                   a_hi | (a_slot + ((ks * R_KSTEP + pass * (C::GROUP_A / 2) + j * C::ACC_A) >> 4));
               mma_bf16_pair(tmem + static_cast<uint32_t>(j * nq), adesc, bdesc, idesc,
-                            (!chain_start || ks > 0 || pass > 0) ? 1u : 0u);
+                            (!chain_start || ks > 0 || pass > 0) ? 1u : 0u, el);
             }
           }
         }
-        mma_commit_pair_mask(empty_o(ss), 0xF);  // all four CTAs wrote into the slot
+        mma_commit_pair_mask(empty_o(ss), 0xF, el);  // all four CTAs wrote into the slot
         if (in_chain == RCHAIN - 1 || s == nsteps - 1) {  // the chain ends
-          mma_commit_pair_mask(acc_full, pair_mask);
+          mma_commit_pair_mask(acc_full, pair_mask, el);
           in_chain = 0;
           ++chain_no;
         } else {
@@ -1614,7 +1616,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (++ss == C::NSS) ss = 0;
       }
       }
-      mma_commit_pair(drain_bar);
+      mma_commit_pair(drain_bar, el);
       drain_wait(drain_bar, 0, 200000000ull);
     }
   } else if (warp < WARP_WORK0) {
@@ -1979,13 +1981,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC + 4);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   // a cluster holds two CTA pairs (cluster ranks 0-1 and 2-3) with the same
   // k rows and the same range of n on consecutive rows of m; the two CTAs of
   // equal rank hold the same rows of the S tile, and each generates half of
   // them and copies that half into its partner (as in the BF16 right sketch)
-  const uint32_t cr = cluster_ctarank();
+  const uint32_t cr = uniform(cluster_ctarank());
   const uint32_t rank = cr & 1u;  // 0 = even CTA of the pair (MMA issuer)
   const uint32_t pairi = cr >> 1;
   const uint32_t lead_rank = cr & ~1u;  // the pair's even CTA
@@ -2025,7 +2027,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   cluster_sync();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform(*tmem_slot);
   const Abort ab{abort_flag, p.status, p.timeout_ns};
   const uint32_t lead_full_o = mapa_shared(full_o(0), lead_rank);
   const uint32_t lead_acc_empty = mapa_shared(acc_empty, lead_rank);
@@ -2053,15 +2055,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
     }
   } else if (warp == WARP_MMA) {
-    if (lane == 0 && leader) {
+    if (leader) {  // the whole warp; one lane issues
+      const uint32_t el = elect_one();
       const uint32_t idesc = idesc_e4m3_f32(256u, static_cast<uint32_t>(nq));
       for (int s = 0; s < nsteps; ++s) {
         const int so = s % C::NSO;
         const int in_chain = s % QCHAIN;
         if (s > 0 && in_chain == 0 &&
-            !mbar_wait(acc_empty, ((s / QCHAIN) - 1) & 1, ab, 0x25, s))
+            !mbar_wait_warp(acc_empty, ((s / QCHAIN) - 1) & 1, ab, 0x25, s))
           break;
-        if (!mbar_wait(full_o(so), (s / C::NSO) & 1, ab, 0x22, s)) break;
+        if (!mbar_wait_warp(full_o(so), (s / C::NSO) & 1, ab, 0x22, s)) break;
         tc_fence_after();
 #pragma unroll
         for (int ks = 0; ks < QK / 32; ++ks) {
@@ -2075,13 +2078,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     static_cast<uint32_t>(ks) * 32u,
                 16u, 1024u);
             mma_e4m3_pair(tmem + static_cast<uint32_t>(j * nq), adesc, bdesc, idesc,
-                          (in_chain > 0 || ks > 0) ? 1u : 0u);
+                          (in_chain > 0 || ks > 0) ? 1u : 0u, el);
           }
         }
-        mma_commit_pair_mask(empty_o(so), 0xF);  // all four CTAs wrote into the slot
-        if (in_chain == QCHAIN - 1 || s == nsteps - 1) mma_commit_pair_mask(acc_full, pair_mask);
+        mma_commit_pair_mask(empty_o(so), 0xF, el);  // all four CTAs wrote into the slot
+        if (in_chain == QCHAIN - 1 || s == nsteps - 1) mma_commit_pair_mask(acc_full, pair_mask, el);
       }
-      mma_commit_pair(drain_bar);
+      mma_commit_pair(drain_bar, el);
       drain_wait(drain_bar, 0, 200000000ull);
     }
   } else if (warp < WARP_WORK0) {

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
   // kSawTiny / kSawNormal of the last four items: the workers are at most
   // three stages, hence three items, ahead of the epilogue
   int* saw = reinterpret_cast<int*>(smem + OFF_MISC + 16);
-  const int warp = threadIdx.x >> 5;
+  const int warp = uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -220,67 +220,67 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
   tc_fence_after();
   pdl_wait();
   pdl_trigger();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform(*tmem_slot);
   const Abort ab{abort_flag, p.status, p.timeout_ns};
   const uint32_t a_part = static_cast<uint32_t>(p.nt / 64) * A_CHUNK;  // one part of A in a slot
   const uint32_t slot_bytes = OFF_A + 3u * a_part;
   const int first_item = static_cast<int>(blockIdx.x), item_step = static_cast<int>(gridDim.x);
 
-  if (warp == 0) {
-    if (lane == 0) {
-      const uint32_t idesc =
-          idesc_bf16_f32(BM, static_cast<uint32_t>(p.nt)) | (1u << 16);  // B is MN-major
-      const uint64_t a_base = smem_desc(sbase, 128u, 256u);
-      const uint64_t b_base = smem_desc_sw128(sbase + OFF_A, A_CHUNK, 1024u);
-      int g = 0, gc = 0, j = 0;
-      bool stop = false;
-      for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
-        const int nsteps = get_item(p, idx).nsteps;
-        int in_chain = 0;
-        for (int s = 0; s < nsteps; ++s, ++g) {
-          const int so = g % SLOTS;
-          if (in_chain == 0 && gc > 0) {
-            // every epilogue warp has read the last chain (and its item's flags)
-            if (!mbar_wait(acc_empty, (gc - 1) & 1, ab, 0x25, gc)) {
-              stop = true;
-              break;
-            }
-            if (s == 0) saw[(j - 1) & 3] = 0;
-          }
-          if (!mbar_wait(full(so), (g / SLOTS) & 1, ab, 0x22, g)) {
+  if (warp == 0) {  // the whole warp; one lane issues
+    const uint32_t el = elect_one();
+    const uint32_t idesc =
+        idesc_bf16_f32(BM, static_cast<uint32_t>(p.nt)) | (1u << 16);  // B is MN-major
+    const uint64_t a_base = smem_desc(sbase, 128u, 256u);
+    const uint64_t b_base = smem_desc_sw128(sbase + OFF_A, A_CHUNK, 1024u);
+    int g = 0, gc = 0, j = 0;
+    bool stop = false;
+    for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+      const int nsteps = get_item(p, idx).nsteps;
+      int in_chain = 0;
+      for (int s = 0; s < nsteps; ++s, ++g) {
+        const int so = g % SLOTS;
+        if (in_chain == 0 && gc > 0) {
+          // every epilogue warp has read the last chain (and its item's flags)
+          if (!mbar_wait_warp(acc_empty, (gc - 1) & 1, ab, 0x25, gc)) {
             stop = true;
             break;
           }
-          tc_fence_after();
-          // offsets are multiples of 16 B below 256 KB: added to the low word
-          const uint64_t a0 = a_base + ((static_cast<uint32_t>(so) * slot_bytes) >> 4);
-          const uint64_t b0 = b_base + ((static_cast<uint32_t>(so) * slot_bytes) >> 4);
+          if (s == 0 && lane == 0) saw[(j - 1) & 3] = 0;
+          __syncwarp();
+        }
+        if (!mbar_wait_warp(full(so), (g / SLOTS) & 1, ab, 0x22, g)) {
+          stop = true;
+          break;
+        }
+        tc_fence_after();
+        // offsets are multiples of 16 B below 256 KB: added to the low word
+        const uint64_t a0 = a_base + ((static_cast<uint32_t>(so) * slot_bytes) >> 4);
+        const uint64_t b0 = b_base + ((static_cast<uint32_t>(so) * slot_bytes) >> 4);
 #pragma unroll
-          for (int ks = 0; ks < 2; ++ks) {
-            auto mma = [&](int sp, int ap, uint32_t col, uint32_t acc) {
-              mma_bf16(tmem + col, a0 + ((sp * S_PART + ks * S_SLAB) >> 4),
-                       b0 + ((static_cast<uint32_t>(ap) * a_part + ks * 2048u) >> 4), idesc, acc);
-            };
-            mma(0, 0, 0u, in_chain > 0 || ks > 0 ? 1u : 0u);
-            mma(0, 1, 256u, s > 0 || ks > 0 ? 1u : 0u);
-            mma(0, 2, 256u, 1u);
-            if (NS == 3) {
-              mma(1, 0, 256u, 1u);
-              mma(1, 1, 256u, 1u);
-              mma(2, 0, 256u, 1u);
-            }
-          }
-          mma_commit(empty(so));
-          if (++in_chain == p.chain || s == nsteps - 1) {
-            mma_commit(acc_full);
-            in_chain = 0;
-            ++gc;
+        for (int ks = 0; ks < 2; ++ks) {
+          auto mma = [&](int sp, int ap, uint32_t col, uint32_t acc) {
+            mma_bf16(tmem + col, a0 + ((sp * S_PART + ks * S_SLAB) >> 4),
+                     b0 + ((static_cast<uint32_t>(ap) * a_part + ks * 2048u) >> 4), idesc, acc, el);
+          };
+          mma(0, 0, 0u, in_chain > 0 || ks > 0 ? 1u : 0u);
+          mma(0, 1, 256u, s > 0 || ks > 0 ? 1u : 0u);
+          mma(0, 2, 256u, 1u);
+          if (NS == 3) {
+            mma(1, 0, 256u, 1u);
+            mma(1, 1, 256u, 1u);
+            mma(2, 0, 256u, 1u);
           }
         }
+        mma_commit(empty(so), el);
+        if (++in_chain == p.chain || s == nsteps - 1) {
+          mma_commit(acc_full, el);
+          in_chain = 0;
+          ++gc;
+        }
       }
-      mma_commit(drain_bar);
-      drain_wait(drain_bar, 0, 200000000ull);
     }
+    mma_commit(drain_bar, el);
+    drain_wait(drain_bar, 0, 200000000ull);
   } else if (warp < W_WORK0) {
     // ---- epilogue: lanes are accumulator rows, main in columns 0 .. nt - 1,
     // cross in 256 .. ----
