@@ -101,7 +101,9 @@ class _Lazy:
     def __getattr__(self, name):
         if _Lazy._lib is None:
             _Lazy._lib = _load()
-        return getattr(_Lazy._lib, name)
+        f = getattr(_Lazy._lib, name)
+        setattr(self, name, f)  # found directly from the next call on
+        return f
 
 
 _lib = _Lazy()

@@ -41,10 +41,10 @@ bool valid_prec(int p) { return p == SK_FP32 || p == SK_BF16X2 || p == SK_FP8E4M
 // where they can)
 size_t workspace_for(const sk_sketch* h, const GemmShape& s, bool least = false) {
   if (h->prec == SK_FP32) {
-    const size_t simt = sk::simt_workspace_bytes(s);
-    if (!sk::tc32_applies(s)) return simt;
     const size_t tc = sk::tc32_workspace_bytes(s);
-    return least && simt < tc ? simt : tc;
+    if (tc != 0 && !least) return tc;
+    const size_t simt = sk::simt_workspace_bytes(s);
+    return tc != 0 && tc < simt ? tc : simt;
   }
   if (h->prec == SK_FP8E4M3) return s.left ? 0 : sk::q8_workspace_bytes(s);
   return sk::tc_workspace_bytes(s, least);
@@ -109,7 +109,8 @@ sk_status apply(sk_sketch* h, const float* A, int64_t m, int64_t n, int64_t lda,
   if (st != SK_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  if (h->prec == SK_FP32 && sk::tc32_applies(s) && h->ws_bytes >= sk::tc32_workspace_bytes(s))
+  const size_t tc32 = h->prec == SK_FP32 ? sk::tc32_workspace_bytes(s) : 0;
+  if (tc32 != 0 && h->ws_bytes >= tc32)
     e = sk::tc32_sketch_left(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);
   else if (h->prec == SK_FP32)  // the CUDA cores; also where a lent buffer is too small
     e = sk::simt_sketch(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);

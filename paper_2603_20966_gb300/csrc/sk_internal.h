@@ -90,6 +90,25 @@ struct GemmShape {
   int64_t P, Q, L;
 };
 
+// The number of splits (at most smax) of a product of `tiles` output tiles
+// that fills whole waves of `units` resident CTAs (or pairs) best: more of
+// them only for 2 % better filled waves, none beyond 4 waves.  Called several
+// times per sketch, so the waves are counted, not divided for.
+inline int64_t best_splits(int64_t tiles, int64_t units, int64_t smax) {
+  int64_t best = 1, waves = 1;
+  double best_fill = -1.0;
+  for (int64_t sp = 1, items = tiles; sp <= smax; ++sp, items += tiles) {
+    if (waves * units < items) waves = (items + units - 1) / units;
+    const double fill = static_cast<double>(items) / static_cast<double>(waves * units);
+    if (fill > best_fill + 0.02) {
+      best_fill = fill;
+      best = sp;
+    }
+    if (items >= 4 * units || best_fill > 0.98) break;  // (nothing is 2 % better)
+  }
+  return best;
+}
+
 // ---- FP32 SIMT form (sk_simt.cu) ----
 size_t simt_workspace_bytes(const GemmShape& s);
 cudaError_t simt_sketch(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
@@ -115,7 +134,7 @@ cudaError_t splitk_reduce_batched(const ReduceDesc* d_desc, int nprob, int64_t m
                                   cudaStream_t st);
 
 // ---- FP32 form of the left sketch on the tensor cores (sk_tc32.cu) ----
-bool tc32_applies(const GemmShape& s);
+// Bytes of its partials, or 0 where the sketch stays on the CUDA cores.
 size_t tc32_workspace_bytes(const GemmShape& s);
 cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
                              float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st);

@@ -2509,18 +2509,7 @@ LeftPlan plan_left(const GemmShape& s) {
   int64_t smax = steps_total / 4;  // at least 128 rows per split
   if (smax > 128) smax = 128;
   if (smax < 1) smax = 1;
-  int64_t best = 1;
-  double best_eff = -1.0;
-  for (int64_t sp = 1; sp <= smax; ++sp) {
-    const int64_t items = tiles * sp;
-    const int64_t waves = (items + units - 1) / units;
-    const double eff = static_cast<double>(items) / static_cast<double>(waves * units);
-    if (eff > best_eff + 0.02) {
-      best_eff = eff;
-      best = sp;
-    }
-    if (items >= 4 * units) break;
-  }
+  const int64_t best = best_splits(tiles, units, smax);
   set_splits(&pl, s, best);
   return pl;
 }

@@ -551,17 +551,7 @@ F32Plan plan_f32(const GemmShape& s, int dist = kGaussian) {
   const int64_t tiles = pl.tiles_p * pl.tiles_q, sms = sm_count();
   const int64_t steps = (s.L + SL - 1) / SL;
   const int64_t smax = std::max<int64_t>(1, std::min<int64_t>(steps / GROUPS, 64));
-  int64_t best = 1;
-  double best_fill = -1.0;
-  for (int64_t sp = 1; sp <= smax; ++sp) {
-    const int64_t items = tiles * sp, waves = (items + sms - 1) / sms;
-    const double fill = static_cast<double>(items) / static_cast<double>(waves * sms);
-    if (fill > best_fill + 0.02) {
-      best_fill = fill;
-      best = sp;
-    }
-    if (items >= 4 * sms) break;
-  }
+  const int64_t best = best_splits(tiles, sms, smax);
   int64_t per = (steps + best - 1) / best;
   pl.chunk = per * SL;
   pl.splits = static_cast<int>((steps + per - 1) / per);
@@ -614,25 +604,24 @@ cudaError_t launch_f32(const CUtensorMap& pmap, const F32Params& p, unsigned gri
 //   64 x 32, 64          21 -> 16 us      1.5e-7 -> 6.7e-8
 //   32 x 512, 512        15.2 -> 17.5 us  (one stage: stays on the CUDA cores)
 // Chains of 11, 19 and 32 stages had errors of 3.4e-7, 5.8e-7 and 8.3e-7.
-bool tc32_applies(const GemmShape& s) {
-  if (!s.left || s.L < 2 * SL) return false;
-  const F32Plan pl = plan_f32(s);
-  // (a k of more than 65535 tiles is refused, as the CUDA-core form does)
-  if (s.P > 65535LL * (s.Q > 128 ? 128 : 256)) return false;
-  // 32-bit item numbers, and strides that a tensor map holds
-  return pl.tiles_p * pl.tiles_q * pl.splits < (int64_t(1) << 31) && s.Q < (int64_t(1) << 31) &&
-         s.P * pl.ldp * 4 < (int64_t(1) << 40);
-}
-
 size_t tc32_workspace_bytes(const GemmShape& s) {
+  if (!s.left || s.L < 2 * SL) return 0;
+  // (a k of more than 65535 tiles is refused, as the CUDA-core form does)
+  if (s.P > 65535LL * (s.Q > 128 ? 128 : 256)) return 0;
   const F32Plan pl = plan_f32(s);
+  // 32-bit item numbers, and strides that a tensor map holds
+  if (pl.tiles_p * pl.tiles_q * pl.splits >= (int64_t(1) << 31) || s.Q >= (int64_t(1) << 31) ||
+      s.P * pl.ldp * 4 >= (int64_t(1) << 40))
+    return 0;
   return static_cast<size_t>(pl.splits) * s.P * pl.ldp * sizeof(float);
 }
 
 cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
                              float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st) {
-  if (ws == nullptr || ws_bytes < tc32_workspace_bytes(s)) return cudaErrorInvalidValue;
   const F32Plan pl = plan_f32(s, h->dist);
+  if (ws == nullptr ||
+      ws_bytes < static_cast<size_t>(pl.splits) * s.P * pl.ldp * sizeof(float))
+    return cudaErrorInvalidValue;
   F32Params p;
   memset(&p, 0, sizeof(p));
   p.A = A;

@@ -12,6 +12,12 @@ import torch
 from . import _native as N
 
 
+def _stream_of(A: torch.Tensor) -> int:
+    """torch's current stream on A's device, as the library takes it: without
+    a Stream object, which costs more than a small sketch's launches."""
+    return torch._C._cuda_getCurrentRawStream(A.get_device())
+
+
 class Sketch:
     def __init__(self, seed: int, dist: int, k: int, precision: int = N.SK_FP32):
         self.handle = N.sk_create(seed, dist, k)
@@ -59,7 +65,7 @@ class Sketch:
         Y = out if out is not None else torch.empty((self.k, n), dtype=torch.float32,
                                                       device=A.device)
         N.sk_apply_left(self.handle, A, m, n, A.stride(0), Y, Y.stride(0),
-                        torch.cuda.current_stream(A.device))
+                        _stream_of(A))
         return Y
 
     def right(self, A: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
@@ -68,7 +74,7 @@ class Sketch:
         Y = out if out is not None else torch.empty((m, self.k), dtype=torch.float32,
                                                       device=A.device)
         N.sk_apply_right(self.handle, A, m, n, A.stride(0), Y, Y.stride(0),
-                         torch.cuda.current_stream(A.device))
+                         _stream_of(A))
         return Y
 
     def nystrom(self, A: torch.Tensor) -> tuple[torch.Tensor, torch.Tensor]:
@@ -79,7 +85,7 @@ class Sketch:
         B = torch.empty((n, ld), dtype=torch.float32, device=A.device)
         C = torch.empty((self.k, ld), dtype=torch.float32, device=A.device)
         N.sk_nystrom(self.handle, A, n, A.stride(0), B, ld, C, ld,
-                     torch.cuda.current_stream(A.device))
+                     _stream_of(A))
         return B[:, :self.k], C[:, :self.k]
 
     def materialize(self, row0: int, col0: int, rows: int, cols: int, fmt: int = N.SK_FP32,
