@@ -543,14 +543,21 @@ F32Plan plan_f32(const GemmShape& s, int dist = kGaussian) {
   F32Plan pl;
   const int64_t chunks = (s.Q + 63) / 64;
   pl.tiles_q = (chunks + NCH - 1) / NCH;
-  pl.nt = static_cast<int>((chunks + pl.tiles_q - 1) / pl.tiles_q) * 64;
   pl.tiles_p = (s.P + BM - 1) / BM;
   pl.ldp = (s.Q + 3) / 4 * 4;
   // splits of m that fill whole waves of CTAs, each at least one stage per
-  // worker group
-  const int64_t tiles = pl.tiles_p * pl.tiles_q, sms = sm_count();
+  // worker group; where the most of them leave SMs idle, narrower tiles (each
+  // generates its S again, but drains sooner: 4096 x 256, k = 64 18.7 -> 16.4
+  // us); more than 64 splits (whose partials the reduction reads) only of
+  // eight stages or more (65536 x 32, k = 64 57 -> 31 us)
+  const int64_t sms = sm_count();
   const int64_t steps = (s.L + SL - 1) / SL;
-  const int64_t smax = std::max<int64_t>(1, std::min<int64_t>(steps / GROUPS, 64));
+  const int64_t smax = std::max<int64_t>(
+      {int64_t{1}, std::min<int64_t>(steps / GROUPS, 64), std::min<int64_t>(steps / 8, sms)});
+  while (pl.tiles_q < chunks && pl.tiles_p * (pl.tiles_q + 1) * smax <= sms) ++pl.tiles_q;
+  pl.nt = static_cast<int>((chunks + pl.tiles_q - 1) / pl.tiles_q) * 64;
+  pl.tiles_q = (chunks * 64 + pl.nt - 1) / pl.nt;
+  const int64_t tiles = pl.tiles_p * pl.tiles_q;
   const int64_t best = best_splits(tiles, sms, smax);
   int64_t per = (steps + best - 1) / best;
   pl.chunk = per * SL;
@@ -595,13 +602,14 @@ cudaError_t launch_f32(const CUtensorMap& pmap, const F32Params& p, unsigned gri
 // The left sketch with at least two stages of m.  Time, and relative
 // Frobenius error against 64 bits, with FP32 FMAs on the CUDA cores and here
 // (Gaussian S; m x n, k):
-//   4096 x 256, 64       39 -> 18 us      2.3e-7 -> 1.5e-7
-//   30011 x 333, 666     644 -> 207 us    5.4e-7 -> 2.5e-7
-//   65536 x 512, 1024    1590 -> 647 us   1.1e-6 -> 2.6e-7
-//   16384 x 100, 300     85 -> 36 us      3.2e-7 -> 2.1e-7
-//   200000 x 16, 16      754 -> 126 us    1.1e-6 -> 2.3e-7
-//   1000 x 1, 1          44 -> 17 us      1.3e-7 -> 2.3e-8
-//   64 x 32, 64          21 -> 16 us      1.5e-7 -> 6.7e-8
+//   4096 x 256, 64       39 -> 15.4 us    2.3e-7 -> 1.5e-7
+//   30011 x 333, 666     644 -> 193 us    5.4e-7 -> 2.5e-7
+//   65536 x 512, 1024    1590 -> 609 us   1.1e-6 -> 2.6e-7
+//   65536 x 32, 64       253 -> 31 us     5.9e-7 -> 3.0e-7
+//   16384 x 100, 300     85 -> 35 us      3.2e-7 -> 2.1e-7
+//   200000 x 16, 16      754 -> 59 us     1.1e-6 -> 3.0e-7
+//   1000 x 1, 1          44 -> 14 us      1.3e-7 -> 2.3e-8
+//   64 x 32, 64          21 -> 13 us      1.5e-7 -> 6.7e-8
 //   32 x 512, 512        15.2 -> 17.5 us  (one stage: stays on the CUDA cores)
 // Chains of 11, 19 and 32 stages had errors of 3.4e-7, 5.8e-7 and 8.3e-7.
 size_t tc32_workspace_bytes(const GemmShape& s) {
