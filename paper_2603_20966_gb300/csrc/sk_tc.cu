@@ -1269,19 +1269,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // BF16 core matrices, hi (512 bytes: 4 of 8 rows x 8 columns) then lo, so a
 // warp converts whole groups with no other warp involved, and the MMA reads
 // hi and lo with 1 KB between 8-row groups.  With no separate staging ring
-// the slots are 32 KB and the ring is 4 stages deep, so up to 128 KB of A per
-// SM are in flight from HBM.  The S tiles have a ring of 8 of their own, so
-// a worker group generates its next S rows while the MMAs of its last stage
-// still read theirs and the A copy that waits for them is on its way
-// (0.993 -> 0.984 ms, Nystrom pair 4.74 -> 4.66 ms).  A stage is 32 columns of n: with 16 (8 slots of
-// 20 KB) every row of the copy was a 64-byte piece of DRAM and the barriers,
-// fences and commits of a stage came twice as
-// often: 65536 x 16384, k = 256 1.174 -> 1.072 ms, the Nystrom pair of a
-// 50,000 x 50,000 matrix, r = 500 5.44 -> 4.96 ms.  Two groups of 8 worker
-// warps instead of four of 4: 1.103 and 5.11 ms (the fences and waits of a
-// stage then stop half the workers at once).  The kernel is persistent: as
-// many clusters as can be resident each take an equal contiguous share of
-// the stages of all blocks, with ring slots,
+// the slots are 32 KB and the ring is 4 stages deep (CfgR: 5 where the
+// generator is cheap), so up to 128 KB of A per SM are in flight from HBM.
+// The S tiles have a ring of their own, so a worker group generates its next
+// S rows while the MMAs of its last stage still read theirs and the A copy
+// that waits for them is on its way (0.993 -> 0.984 ms, Nystrom pair 4.74 ->
+// 4.66 ms).  A stage is 32 columns of n: with 16 (8 slots of 20 KB) every row
+// of the copy was a 64-byte piece of DRAM and the barriers, fences and
+// commits of a stage came twice as often: 65536 x 16384, k = 256 1.174 ->
+// 1.072 ms, the Nystrom pair of a 50,000 x 50,000 matrix, r = 500 5.44 ->
+// 4.96 ms.  Two groups of 8 worker warps instead of four of 4: 1.103 and
+// 5.11 ms (the fences and waits of a stage then stop half the workers at
+// once).  The kernel is persistent: as many clusters as can be resident each
+// take an equal contiguous share of the stages of all blocks, with ring slots,
 // barrier phases and chains counted across items, so the next item's copies
 // and S tiles are under way while the last chain of the previous one drains.
 // ---------------------------------------------------------------------------
@@ -1289,13 +1289,19 @@ constexpr int RK = 32;               // contracted length per stage of the right
 constexpr int RSTEPS = RK / BK;      // MMA K steps per right stage
 constexpr int RCHAIN = CHAIN / RSTEPS;  // right stages per accumulation chain
 
+// DEEP_A: a fifth A tile in the ring for four S tiles less.  Rademacher and
+// uniform workers spend their time waiting for A (65536 x 16384, k = 256
+// Rademacher 0.876 -> 0.831 ms, 20011 x 3071, k = 100 uniform 63 -> 60 us);
+// Gaussian ones generate and want the S tiles (0.979 against 1.000 ms).
+template <bool DEEP_A>
 struct CfgR {
   static constexpr int ROWS = 256;  // rows of A per CTA (two 128-row accumulators)
   static constexpr int NGROUPS = 4;
   static constexpr int GROUP_WARPS = NUM_WORK_WARPS / NGROUPS;
   static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
-  static constexpr int NS = 4;                        // A tiles in the ring
-  static constexpr int NSS = 8;                       // S tiles
+  static constexpr int NS = DEEP_A ? 5 : 4;           // A tiles in the ring
+  static constexpr int NSS = DEEP_A ? 4 : 8;          // S tiles
+  static constexpr int NE = 8;                        // "MMAs completed" barriers
   static constexpr uint32_t OPA = RK * ROWS * 4;      // FP32 A tile = its hi and lo halves
   static constexpr uint32_t ACC_A = OPA / 2;          // hi + lo of one 128-row accumulator
   static constexpr uint32_t GROUP_A = 8 * RK * 4;     // one 8-row group, FP32 = hi + lo
@@ -1308,17 +1314,21 @@ struct CfgR {
   static constexpr uint32_t EPI_BYTES = DRAIN_TILE;
   static constexpr uint32_t OFF_EPI = OFF_S + NSS * OPS;
   static constexpr uint32_t OFF_BAR = OFF_EPI + NUM_EPI_WARPS * EPI_BYTES;
-  // per A slot: A landed, operands ready; per S slot: stage read by both
-  // pairs' MMAs, S rows received from the partner CTA; then the accumulator
-  // and drain barriers
-  static constexpr uint32_t NUM_BARS = 2 * NS + 2 * NSS + 3;
+  // per A slot: A landed, operands ready; per stage of NE: read by both
+  // pairs' MMAs; per S slot: S rows received from the partner CTA; then the
+  // accumulator and drain barriers
+  static constexpr uint32_t NUM_BARS = 2 * NS + NE + NSS + 3;
   static constexpr uint32_t OFF_MISC = OFF_BAR + NUM_BARS * 8;
   static constexpr uint32_t SMEM = OFF_MISC + 16 + 1024;
   static_assert(SMEM <= 227 * 1024, "shared memory budget");
-  static_assert(NGROUPS <= NS && NS <= NSS, "worker groups vs ring depths");
+  static_assert(NGROUPS <= NSS && NSS <= NE && NS <= NE, "worker groups vs ring depths");
   static_assert(OPA % 1024 == 0 && OPS % 1024 == 0, "slots on 1 KB boundaries");
   static_assert(OFF_EPI % 1024 == 0, "epilogue tiles on swizzle-atom boundaries");
 };
+
+constexpr int R_ROWS = CfgR<false>::ROWS;
+constexpr uint32_t R_SMEM =
+    CfgR<true>::SMEM > CfgR<false>::SMEM ? CfgR<true>::SMEM : CfgR<false>::SMEM;
 
 // Operand layout of a right stage: K-major core matrices (8 rows x 8
 // columns, 128 bytes, row r at 16 r), the four of an 8-row group of the 32
@@ -1326,7 +1336,7 @@ struct CfgR {
 // GROUP_A apart (A).  One K step is two core matrices: 256 bytes.
 constexpr uint32_t R_KSTEP = 256;
 __device__ __forceinline__ uint32_t right_s_off(uint32_t row, uint32_t chunk) {
-  return (row >> 3) * CfgR::GROUP_S + chunk * 128u + (row & 7u) * 16u;
+  return (row >> 3) * CfgR<false>::GROUP_S + chunk * 128u + (row & 7u) * 16u;
 }
 
 struct TcRightParams {
@@ -1416,7 +1426,7 @@ template <int DIST>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_sketch_bf16x2_right(const __grid_constant__ CUtensorMap tmapA,
                           const __grid_constant__ CUtensorMap tmapP, const TcRightParams p) {
-  using C = CfgR;
+  using C = CfgR<DIST != kGaussian>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -1426,12 +1436,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // operands of the stage are ready; empty_o: both pairs' MMAs have read
   // what this CTA wrote for the stage (here and, S rows, in its partner);
   // s_recv: the S rows the partner CTA copies into the slot have landed.
-  // full_b and full_o count stages in the ring of A, the others in that of S
+  // full_b and full_o count stages in the ring of A, s_recv in that of S,
+  // empty_o in one of NE stages (the slot of A or S that stage g reuses is
+  // free once the barrier of stage g - NS or g - NSS says so)
   auto full_b = [&](int i) { return bar0 + 8u * i; };
   auto full_o = [&](int i) { return bar0 + 8u * (C::NS + i); };
   auto empty_o = [&](int i) { return bar0 + 8u * (2 * C::NS + i); };
-  auto s_recv = [&](int i) { return bar0 + 8u * (2 * C::NS + C::NSS + i); };
-  const uint32_t acc_full = bar0 + 8u * (2 * C::NS + 2 * C::NSS);
+  auto s_recv = [&](int i) { return bar0 + 8u * (2 * C::NS + C::NE + i); };
+  const uint32_t acc_full = bar0 + 8u * (2 * C::NS + C::NE + C::NSS);
   const uint32_t acc_empty = acc_full + 8u;
   const uint32_t drain_bar = acc_full + 16u;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC);
@@ -1489,8 +1501,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_init(full_b(i), 1);
       mbar_init(full_o(i), C::GROUP_WARPS * 2);  // one worker group of each CTA of the pair
     }
-    for (int i = 0; i < C::NSS; ++i) {
+    for (int i = 0; i < C::NE; ++i)
       mbar_init(empty_o(i), 2);  // the MMAs of both pairs read what this CTA wrote
+    for (int i = 0; i < C::NSS; ++i) {
       mbar_init(s_recv(i), 1);   // the receiving group's expect-tx, plus the copy's bytes
     }
     mbar_init(acc_full, 1);
@@ -1533,7 +1546,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         for (int s = 0; s < it.nsteps; ++s, ++g) {
           const int so = g % C::NS;
           const int v = g - C::NS;  // the stage that had this slot: both pairs have read it
-          if (v >= 0 && !mbar_wait(empty_o(v % C::NSS), (v / C::NSS) & 1, ab, 0x13, g)) {
+          if (v >= 0 && !mbar_wait(empty_o(v % C::NE), (v / C::NE) & 1, ab, 0x13, g)) {
             stop = true;
             break;
           }
@@ -1601,7 +1614,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
           }
         }
-        mma_commit_pair_mask(empty_o(ss), 0xF, el);  // all four CTAs wrote into the slot
+        mma_commit_pair_mask(empty_o(g % C::NE), 0xF, el);  // all four CTAs wrote into the slot
         if (in_chain == RCHAIN - 1 || s == nsteps - 1) {  // the chain ends
           mma_commit_pair_mask(acc_full, pair_mask, el);
           in_chain = 0;
@@ -1745,7 +1758,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const int ss = g % C::NSS;
       // both pairs' MMAs have read what this CTA wrote into S slot `ss` (here
       // and in its partner) last time
-      bool ok = g < C::NSS || mbar_wait(empty_o(ss), ((g / C::NSS) & 1) ^ 1, ab, 0x43, g);
+      const int v = g - C::NSS;  // the stage that had this S slot
+      bool ok = v < 0 || mbar_wait(empty_o(v % C::NE), (v / C::NE) & 1, ab, 0x43, g);
       if (!__all_sync(0xffffffffu, ok)) {
         stop = true;
         break;
@@ -2787,13 +2801,13 @@ cudaError_t set_smem_attr_right() {
   static bool done = false;
   if (done) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(k_sketch_bf16x2_right<kGaussian>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, CfgR::SMEM);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, R_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_sketch_bf16x2_right<kRademacher>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, CfgR::SMEM);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, R_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_sketch_bf16x2_right<kUniform>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, CfgR::SMEM);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, R_SMEM);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -2820,7 +2834,7 @@ Plan plan_right(const GemmShape& s, int cluster = 4) {
   pl.nt = s.Q > 256 ? 256 : static_cast<int>((s.Q + 31) / 32 * 32);
   pl.tmem_cols = 32;
   while (pl.tmem_cols < 2 * pl.nt) pl.tmem_cols *= 2;
-  const int64_t rows = static_cast<int64_t>(cluster) * CfgR::ROWS;  // rows of m per cluster
+  const int64_t rows = static_cast<int64_t>(cluster) * R_ROWS;  // rows of m per cluster
   pl.tiles_p = (s.P + rows - 1) / rows * cluster;                  // CTAs along m
   pl.tiles_q = (s.Q + pl.nt - 1) / pl.nt;
   int64_t slots = cluster == 4 ? quad_slots() : pair_slots();
@@ -2908,7 +2922,7 @@ int64_t quad_slots() {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_config<true>(&cfg, attr, dim3(4, 1, 1), nullptr, 4);
-  cfg.dynamicSmemBytes = CfgR::SMEM;
+  cfg.dynamicSmemBytes = R_SMEM;
   int clusters = 0;
   if (cudaOccupancyMaxActiveClusters(&clusters, k_sketch_bf16x2_right<kGaussian>, &cfg) !=
           cudaSuccess ||
@@ -2924,7 +2938,7 @@ cudaError_t launch_right(const CUtensorMap& map, const CUtensorMap& pmap, const 
                          dim3 grid, cudaStream_t st) {
   cudaError_t e = set_smem_attr_right();
   if (e != cudaSuccess) return e;
-  return launch_overlapped(k_sketch_bf16x2_right<DIST>, grid, dim3(NTHREADS), CfgR::SMEM, st, 4,
+  return launch_overlapped(k_sketch_bf16x2_right<DIST>, grid, dim3(NTHREADS), R_SMEM, st, 4,
                            map, pmap, p);
 }
 
@@ -3024,11 +3038,11 @@ __global__ void __launch_bounds__(256)
   pdl_wait();
   pdl_trigger();
   if (ty >= tyn) return;
-  const int64_t mblocks = (P + 4 * CfgR::ROWS - 1) / (4 * CfgR::ROWS);
+  const int64_t mblocks = (P + 4 * R_ROWS - 1) / (4 * R_ROWS);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * tyn;
   for (int64_t mb = blockIdx.y; mb < mblocks; mb += gridDim.y) {
-    const int64_t r0 = mb * (4 * CfgR::ROWS) + static_cast<int64_t>(blockIdx.x) * tyn + ty;
-    const int64_t r1 = min(P, (mb + 1) * (4 * CfgR::ROWS));
+    const int64_t r0 = mb * (4 * R_ROWS) + static_cast<int64_t>(blockIdx.x) * tyn + ty;
+    const int64_t r1 = min(P, (mb + 1) * (4 * R_ROWS));
     for (int64_t g = tx; g < gpr; g += txn) {
       const int64_t c = g * W;
       const int64_t blk = mb * tiles_q + c / nq;
@@ -3105,7 +3119,7 @@ cudaError_t tc_sketch_right(const sk_sketch* h, const GemmShape& s, const float*
   CUtensorMap map;
   // A[m x n]: n innermost; one box = 32 columns of n x 256 rows of m, each
   // 128-byte row with the 128-byte swizzle (the in-place split's lane map)
-  if (!encode_map(&map, A, s.P, s.L, lda, RK, CfgR::ROWS, CU_TENSOR_MAP_SWIZZLE_128B))
+  if (!encode_map(&map, A, s.P, s.L, lda, RK, R_ROWS, CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
   TcRightParams p;
   p.P = s.P;
@@ -3148,7 +3162,7 @@ cudaError_t tc_sketch_right(const sk_sketch* h, const GemmShape& s, const float*
   const int tyn = 256 / txn;
   // one pass: 4 rows a thread, or 1 of many segments
   const int rows = tyn * (rs.zmax >= kManySegments ? 1 : 4);
-  const dim3 rgrid(static_cast<unsigned>((4 * CfgR::ROWS + rows - 1) / rows),
+  const dim3 rgrid(static_cast<unsigned>((4 * R_ROWS + rows - 1) / rows),
                    static_cast<unsigned>(std::min<int64_t>(mblocks, 65535)));
   count_launches(1);
   return launch_overlapped(vec ? k_reduce_segments<4> : k_reduce_segments<1>, rgrid, dim3(256), 0,
