@@ -38,7 +38,9 @@
  *    a bounds check) are recorded in a per-handle status word that
  *    sk_stream_status() reads.
  *  - Determinism: identical (seed, dist, k, precision, A) give bit-identical
- *    Y on the same GPU model, independent of stream, batch or serving mix.
+ *    Y on the same GPU model, independent of stream, batch or serving mix
+ *    (SK_FP32 left sketches: of those that run on the same cores, see
+ *    sk_set_workspace).
  *  - A handle may be used from one host thread at a time.
  */
 #ifndef SKETCH_H_
@@ -183,9 +185,10 @@ sk_status sk_apply_right_e4m3(sk_handle h, const uint8_t* Aq, const int32_t* row
  * SK_EUNSUPPORTED), with the same argument meaning and layout.  Its split-K
  * partials live in a 16 MiB array compiled into the library, which every GPU
  * that loads the library holds until the process exits.  Problems whose
- * partials would exceed it -- splits * k * n * 4 bytes > 16 MiB, with
- * sk_workspace_size(h, 0, m, n) reporting that byte count -- are rejected
- * with SK_EUNSUPPORTED before anything is enqueued.  Every call looks up the
+ * partials on the CUDA cores would exceed it -- splits * k * n * 4 bytes
+ * > 16 MiB, of which sk_workspace_size(h, 0, m, n) is an upper bound -- are
+ * rejected with SK_EUNSUPPORTED before anything is enqueued; those whose
+ * partials on the tensor cores fit it run there, the others on the CUDA cores.  Every call looks up the
  * current device's address of the array (cudaGetSymbolAddress, which
  * allocates nothing), so the address stays right after a cudaDeviceReset;
  * on a device's first call the CUDA runtime may load the library's device
@@ -227,7 +230,11 @@ sk_status sk_materialize(sk_handle h, int64_t row0, int64_t col0, int64_t rows, 
  * sk_set_workspace lends the handle a caller-owned device buffer of `bytes`
  * (16-byte aligned; NULL/0 returns to handle-owned scratch, which the
  * handle allocates with cudaMalloc on first need and frees in sk_destroy).
- * A lent buffer must stay valid until every call that used it completed. */
+ * A lent buffer must stay valid until every call that used it completed.
+ * SK_FP32 left sketches run on the tensor cores where the buffer holds their
+ * partials, which the size above does; a smaller one is taken as long as it
+ * holds the partials of the CUDA cores' form, which then runs (also in a
+ * server whose budget holds no more, and in sk_apply_left_noalloc). */
 sk_status sk_workspace_size(sk_handle h, int side, int64_t m, int64_t n, size_t* bytes);
 sk_status sk_set_workspace(sk_handle h, void* ptr, size_t bytes);
 

@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <new>
 
@@ -109,11 +110,8 @@ sk_status apply(sk_sketch* h, const float* A, int64_t m, int64_t n, int64_t lda,
   if (st != SK_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  const size_t tc32 = h->prec == SK_FP32 ? sk::tc32_workspace_bytes(s) : 0;
-  if (tc32 != 0 && h->ws_bytes >= tc32)
-    e = sk::tc32_sketch_left(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);
-  else if (h->prec == SK_FP32)  // the CUDA cores; also where a lent buffer is too small
-    e = sk::simt_sketch(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);
+  if (h->prec == SK_FP32)
+    e = sk::fp32_sketch(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);
   else if (h->prec == SK_FP8E4M3)
     e = sk::q8_sketch_right(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);
   else
@@ -317,6 +315,8 @@ sk_status sk_workspace_size(sk_handle h, int side, int64_t m, int64_t n, size_t*
     s.P = m; s.Q = h->k; s.L = n;
   }
   *bytes = workspace_for(h, s);
+  // (the FP32 form: enough for either of its kernels)
+  if (h->prec == SK_FP32) *bytes = std::max(*bytes, sk::simt_workspace_bytes(s));
   return SK_OK;
 }
 

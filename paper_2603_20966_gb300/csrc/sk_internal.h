@@ -139,6 +139,12 @@ size_t tc32_workspace_bytes(const GemmShape& s);
 cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
                              float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st);
 
+// The FP32 form: the tensor cores where the workspace holds their partials,
+// else the CUDA cores.  Every entry point goes through it, so that a sketch
+// has the same bits alone, served and without allocation.
+cudaError_t fp32_sketch(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
+                        float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st);
+
 // ---- batches of left sketches on the tensor cores (sk_tc.cu) ----
 struct BatchMember {
   uint64_t seed;

@@ -465,7 +465,7 @@ cudaError_t sk_server::launch_items(Lane* ln, const std::vector<StepItem>& items
     s.P = it.mb.k;
     s.Q = it.mb.n;
     s.L = it.mb.m;
-    e = sk::simt_sketch(&h, s, it.mb.A, it.mb.lda, it.mb.Y, it.mb.ldy, it.simt_part,
+    e = sk::fp32_sketch(&h, s, it.mb.A, it.mb.lda, it.mb.Y, it.mb.ldy, it.simt_part,
                         it.simt_bytes, ln->st);
   }
   if (e == cudaSuccess)
@@ -728,7 +728,13 @@ sk_status sk_server_submit(sk_server_handle s, sk_handle h, const float* A, int6
     // a readable source is split on admission; a pageable one is copied first
     r.a_bytes = r.src_dev ? 0 : a_copy;
   } else {
-    r.ws_bytes = round_up(sk::simt_workspace_bytes(sh), kAlign);
+    const uint64_t y = round_up(static_cast<uint64_t>(h->k) * r.ldp * sizeof(float), kAlign);
+    const uint64_t simt = round_up(sk::simt_workspace_bytes(sh), kAlign);
+    r.ws_bytes = round_up(sk::tc32_workspace_bytes(sh), kAlign);
+    // the CUDA cores' form where that is the only one, or the only one that
+    // the budget holds
+    if (r.ws_bytes == 0 || (a_copy + r.ws_bytes + y > s->pool.size() && simt < r.ws_bytes))
+      r.ws_bytes = simt;
     r.a_bytes = a_copy;
   }
   r.work_bytes = r.a_bytes + r.ws_bytes;

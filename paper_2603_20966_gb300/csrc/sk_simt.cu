@@ -557,7 +557,7 @@ extern "C" sk_status sk_apply_left_noalloc(sk_handle h, const float* A, int64_t 
   void* scratch = nullptr;
   cudaError_t e = sk::static_scratch_address(&scratch);
   if (e == cudaSuccess)
-    e = sk::simt_sketch(h, s, A, lda, Y, ldy, scratch, sk::kStaticScratchBytes,
+    e = sk::fp32_sketch(h, s, A, lda, Y, ldy, scratch, sk::kStaticScratchBytes,
                         static_cast<cudaStream_t>(stream));
   return sk::status_from_cuda(e);
 }

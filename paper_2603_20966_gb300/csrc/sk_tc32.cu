@@ -154,25 +154,30 @@ __device__ __forceinline__ void split3(float2 x, uint32_t (&w)[3]) {
 }
 
 // A row of an item's tile in FP32 FMAs, for a tile of A too small in
-// magnitude to split (rare: all of it below 2^-100).
+// magnitude to split (rare: all of it below 2^-100), W columns per generated
+// entry.
 __device__ __noinline__ void slow_item(const F32Params& p, int64_t row, int64_t q0, int64_t q1,
                                        int64_t l0, int64_t l1, float* out) {
+  constexpr int W = 16;
   const PhiloxKey key{p.rk.k[0], p.rk.k[1]};
-  for (int64_t c = q0; c < q1; c += 8) {
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const int nc = static_cast<int>(min(static_cast<int64_t>(8), q1 - c));
+  for (int64_t c = q0; c < q1; c += W) {
+    float acc[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) acc[j] = 0.0f;
+    const int nc = static_cast<int>(min(static_cast<int64_t>(W), q1 - c));
     for (int64_t l = l0; l < l1; l += 4) {
       const float4 g = gen4(p.dist, key, static_cast<uint32_t>(row), static_cast<uint32_t>(l));
-      const float gg[4] = {g.x, g.y, g.z, g.w};
-      for (int i = 0; i < 4 && l + i < l1; ++i) {
+      const int nl = static_cast<int>(min(static_cast<int64_t>(4), l1 - l));
+      for (int i = 0; i < nl; ++i) {
+        const float gi = i == 0 ? g.x : i == 1 ? g.y : i == 2 ? g.z : g.w;
         const float* a = p.A + (l + i) * p.lda + c;
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (j < nc) acc[j] = __fmaf_rn(gg[i], a[j], acc[j]);
+        for (int j = 0; j < W; ++j)
+          if (j < nc) acc[j] = __fmaf_rn(gi, __ldg(a + j), acc[j]);
       }
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+    for (int j = 0; j < W; ++j)
       if (j < nc) out[c + j] = acc[j];
   }
 }
@@ -661,6 +666,14 @@ cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float
   if (e != cudaSuccess) return e;
   count_launches(1);
   return splitk_reduce(p.part, pl.splits, s.P, s.Q, pl.ldp, h->scale, Y, ldy, st);
+}
+
+cudaError_t fp32_sketch(const sk_sketch* h, const GemmShape& s, const float* A, int64_t lda,
+                        float* Y, int64_t ldy, void* ws, size_t ws_bytes, cudaStream_t st) {
+  const size_t tc = tc32_workspace_bytes(s);
+  if (tc != 0 && ws != nullptr && ws_bytes >= tc)
+    return tc32_sketch_left(h, s, A, lda, Y, ldy, ws, ws_bytes, st);
+  return simt_sketch(h, s, A, lda, Y, ldy, ws, ws_bytes, st);
 }
 
 }  // namespace sk

@@ -104,3 +104,14 @@ def test_lent_workspaces(P, orc, k, m, n):
             assert S.status() == 0
             assert rel_frob(Y.cpu().numpy(), ref) <= TOL
         P.sk_set_workspace(S.handle, None, 0)
+
+
+def test_same_bits_served_and_without_allocation(P):
+    k, m, n = 70, 3001, 52
+    A = _A(m, n, 8).cuda()
+    with P.Sketch(7, G, k, P.SK_FP32) as S, P.Server(1 << 28) as server:
+        Y, Z = S.left(A), torch.empty((k, n), dtype=torch.float32, device="cuda")
+        P._native.sk_apply_left_noalloc(S.handle, A, m, n, n, Z, n)
+        W = server.result(server.submit(S, A))
+        assert S.status() == 0
+        assert torch.equal(Y, Z) and torch.equal(Y, W)
