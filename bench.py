@@ -744,7 +744,14 @@ def run_ours(args):
 
     pk, pk_kind = peaks()
     avg_kernel_s = statistics.mean(kernel_ms) * 1e-3
-    if form == P.SK_FP32:
+    if form == P.SK_FP32 and side == "left":
+        # three BF16 values per FP32 operand: six BF16 MMA passes, three for Rademacher S
+        passes = statistics.mean(3 if d == P.SK_RADEMACHER else 6 for d in dists)
+        peak = pk["bf16_tflops"]
+        roof = {"bound": "tensor", "achieved": passes * flops_per_sketch / avg_kernel_s / 1e12,
+                "peak": peak, "unit": "TFLOP/s", "peak_kind": f"{pk_kind} bf16 burst",
+                "note": f"achieved counts the {passes} BF16 MMA passes per sketch"}
+    elif form == P.SK_FP32:
         # FP32 FMA pipe: 152 SMs x 128 lanes x 2 flop x max SM clock
         peak = 152 * 128 * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
         roof = {"bound": "alu", "achieved": flops_per_sketch / avg_kernel_s / 1e12, "peak": peak,
