@@ -244,7 +244,7 @@ def generator_floor(dist: int, entries: float, sm_mhz: float, sms: int):
 
 def fp32_comparison(P, A, m, n, k, dists, Ys, stream, steps, ncols=32):
     """The metric's comparison: the same left-sketch step in the plain FP32
-    form (FP32 FMA on the CUDA cores), timed with CUDA events, and the error
+    form (three BF16 values per FP32 operand), timed with CUDA events, and the error
     of both forms against FP64 products of their own S (g for FP32, bf16(g)
     for BF16 split-A, materialized by the library in row blocks of A) over
     `ncols` evenly spaced columns of Y."""
@@ -874,7 +874,8 @@ def run_ours(args):
                                "against FP64 products with each form's own S (g for FP32, "
                                "bf16(g) for BF16 split-A) materialized by the library; "
                                "tolerance 1e-5",
-                   "fp32_form": "FP32 FMA on the CUDA cores, S generated in shared memory"}
+                   "fp32_form": "FP32 operands as sums of three BF16 values on the tensor "
+                                "cores, S generated in shared memory"}
     if roof.get("bound") == "tensor":
         clk_mhz = (clk or {}).get("sm_mhz") or pk.get("sm_max_mhz", 2070.0)
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
