@@ -518,10 +518,13 @@ __device__ __forceinline__ void gen_stage(uint8_t* sdst, const ItemGeo& g, const
 #pragma unroll
     for (int slab = 0; slab < KSTEPS; ++slab)
       pc[slab] = philox_col(key, j0 + 4u * static_cast<uint32_t>(slab));
-    // two tasks in flight per thread: full unrolling of the 8 Philox +
-    // Box-Muller tasks made the loop too large for the instruction cache
-    // (11 % slower on the Gaussian sketch)
-#pragma unroll 1
+    // two tasks in flight per thread (four in batches, whose register-stepped
+    // keys leave longer chains: batch of 256 4.830 -> 4.799 ms; 2^20 x 512,
+    // k = 2048 with launch-parameter keys 3.95 -> 3.97): full unrolling of the
+    // 8 Philox + Box-Muller tasks made the loop too large for the instruction
+    // cache (11 % slower on the Gaussian sketch)
+    constexpr int ROWS_AT_ONCE = std::is_same<K, PhiloxKey>::value ? 2 : 1;
+#pragma unroll ROWS_AT_ONCE
     for (int i = 0; i < NPASS; ++i) {
       const int64_t grow = row0 + static_cast<int64_t>(RSTEP) * i;
       const bool rv = grow < g.P;
