@@ -6,6 +6,8 @@
 // regenerates the tile of the random operand it is about to consume
 // straight into shared memory, so the random matrix is never written to or
 // read from device memory.  Accumulation is FP32 FMA in registers.
+// Left sketches run here only where sk_tc32.cu's form does not apply (fewer
+// than 64 rows of A, or a workspace that holds only these partials).
 #include <cuda_runtime.h>
 
 #include <algorithm>
