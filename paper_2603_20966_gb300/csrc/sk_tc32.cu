@@ -173,7 +173,7 @@ __device__ __noinline__ void slow_item(const F32Params& p, int64_t row, int64_t 
         const float* a = p.A + (l + i) * p.lda + c;
 #pragma unroll
         for (int j = 0; j < W; ++j)
-          if (j < nc) acc[j] = __fmaf_rn(gi, __ldg(a + j), acc[j]);
+          if (j < nc) acc[j] = __fmaf_rn(gi, a[j], acc[j]);
       }
     }
 #pragma unroll
@@ -413,6 +413,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
         for (int half = 0; half < 2; ++half) {
           // this warp's rows 16 half + 2 w, + 1 of the stage, columns 2 lane,
           // + 1 of each chunk, in flight while the S rows are generated
+          // (ordinary loads: the kernel before this one may have written A while
+          // this one was already resident)
           float2 x[2][NCH];
 #pragma unroll
           for (int j2 = 0; j2 < 2; ++j2) {
@@ -425,11 +427,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
               if (c < nfull) {
                 const float* src = row + 2 * lane + 64 * c;
                 if (p.vec2)
-                  x[j2][c] = __ldg(reinterpret_cast<const float2*>(src));
+                  x[j2][c] = *reinterpret_cast<const float2*>(src);
                 else
-                  x[j2][c] = f2(__ldg(src), __ldg(src + 1));
+                  x[j2][c] = f2(src[0], src[1]);
               } else if (c < nconv) {
-                x[j2][c] = f2(__ldg(row + edge0), __ldg(row + edge1));
+                x[j2][c] = f2(row[edge0], row[edge1]);
               }
             }
           }
