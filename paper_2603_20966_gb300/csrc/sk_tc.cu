@@ -127,9 +127,11 @@ template <bool PAIR, bool NARROW = false, bool SRING = false>
 struct Cfg {
   static constexpr int COLS = NT_MAX / (PAIR ? 2 : 1) / (NARROW ? 2 : 1);  // most A columns per CTA
   // Worker groups take turns on successive stages.  A group that starts
-  // stage s has finished stage s - NGROUPS, so waits never run more than one
-  // barrier phase ahead (the parity test would alias) as long as
-  // NGROUPS <= NSO.
+  // stage s has finished stage s - NGROUPS and knows that the MMAs of stage
+  // s - NSS have completed, so its waits on barriers of the S ring never run
+  // more than one phase ahead (the parity test would alias) as long as
+  // NGROUPS <= NSS.  Before a wait on a barrier of a shorter A ring it has to
+  // see the MMAs of stage s - NSO completed too (see the workers' loop).
   static constexpr int NGROUPS = PAIR || NARROW ? 4 : 2;
   static constexpr int GROUP_WARPS = NUM_WORK_WARPS / NGROUPS;
   static constexpr int GROUP_THREADS = 32 * GROUP_WARPS;
@@ -1218,8 +1220,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const bool wconv = (DIST == kRademacher || DIST == kMixed) && PAIR &&
                            ig.pr->conv_inline && (DIST != kMixed || ig.dist == kRademacher);
         if ((!EC && !SRING) || wconv) {  // otherwise the A tile is certified by others
+          // With a separate S ring a group is released NSS stages after its
+          // slot of S, and (behind an item whose A it did not wait for) the A
+          // tile of stage g - NSO may still be on its way: full_b is then a
+          // whole phase behind and the parity test below would let the group
+          // split a slot that holds another stage.  The MMAs of that stage
+          // come first; the copy awaited below started behind them, so this
+          // adds nothing to the wait (batch of 256: 4.86 ms).
+          const int v = g - C::NSO;
+          ok = !SRING || v < 0 || mbar_wait(empty_o(v % C::NSS), (v / C::NSS) & 1, ab, 0x47, g);
           // this CTA's split A tile of the stage has landed
-          ok = mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x40, g);
+          ok = ok && mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x40, g);
           if (!__all_sync(0xffffffffu, ok)) {
             stop = true;
             break;
