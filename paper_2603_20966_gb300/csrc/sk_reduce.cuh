@@ -40,8 +40,7 @@ __device__ __forceinline__ void store_columns(float* row, int64_t c, int64_t Q, 
 
 // Adds `N` partials, all loaded before the first is added.
 template <int N, class V>
-__device__ __forceinline__ const float* add_run(V& s, const float* __restrict__ p,
-                                                int64_t zstride) {
+__device__ __forceinline__ const float* add_run(V& s, const float* p, int64_t zstride) {
   V v[N];
 #pragma unroll
   for (int u = 0; u < N; ++u) v[u] = *reinterpret_cast<const V*>(p + u * zstride);
@@ -53,7 +52,7 @@ __device__ __forceinline__ const float* add_run(V& s, const float* __restrict__ 
 // p[0] + p[zstride] + ... (n terms, in that order), eight loads in flight: a
 // thread's sum is otherwise a chain of n loads, each waiting for the L2.
 template <class V>
-__device__ __forceinline__ V sum_partials(const float* __restrict__ p, int64_t zstride, int n) {
+__device__ __forceinline__ V sum_partials(const float* p, int64_t zstride, int n) {
   V s;
   set_zero(s);
   int z = 0;

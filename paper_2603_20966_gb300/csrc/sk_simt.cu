@@ -277,10 +277,14 @@ __global__ void __launch_bounds__(TPB, 1) k_sketch_fp32_simt(SimtParams p) {
 // 16 bytes per load where rows allow it and has 8 loads in flight
 // (sum_partials).  FP8 right sketch 65536 x 16384, k = 256 (5 partials of
 // 67 MB): 1.503 -> 1.474 ms for the whole call; no change on small outputs.
+// The partials are still being written while this kernel is already resident
+// (launch_overlapped), so they are no __restrict__ parameter, which would
+// promise data that is constant for the kernel's whole life and allow
+// read-only loads, before pdl_wait too.
 template <int W>
 __global__ void __launch_bounds__(256)
-    k_splitk_reduce(const float* __restrict__ part, int splits, int64_t groups, int64_t gpr,
-                    int64_t Q, float scale, float* __restrict__ Y, int64_t ldy) {
+    k_splitk_reduce(const float* part, int splits, int64_t groups, int64_t gpr, int64_t Q,
+                    float scale, float* Y, int64_t ldy) {
   using V = typename std::conditional<W == 4, float4, float>::type;
   const int64_t zstride = groups * W;
   pdl_wait();
@@ -300,7 +304,7 @@ __global__ void __launch_bounds__(256)
 // 256 problems of m in [1024, 65536], n in [32, 512]: 5.34 -> 5.20 ms for the
 // whole batch, against one column and one load in flight per thread.
 __global__ void __launch_bounds__(256)
-    k_splitk_reduce_batched(const ReduceDesc* __restrict__ desc) {
+    k_splitk_reduce_batched(const ReduceDesc* desc) {
   pdl_wait();
   const ReduceDesc d = desc[blockIdx.y];
   const int64_t gpr = d.ldp / 4;

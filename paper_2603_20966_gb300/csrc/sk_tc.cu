@@ -3036,12 +3036,13 @@ RightSegPlan plan_right_seg(const GemmShape& s) {
 // 65536 x 16384, k = 256 1.210 -> 1.170 ms, 20011 x 3071, k = 100 85 ->
 // 69 us), 8 segments of one row at a time when into many, as for small ones
 // (2617 x 345, k = 167, 11 segments: 37 -> 18 us with the padded rows below).
+// `part` is no __restrict__ parameter for k_splitk_reduce's reason.
 constexpr int kManySegments = 8;
 template <int W>
 __global__ void __launch_bounds__(256)
-    k_reduce_segments(const float* __restrict__ part, int64_t P, int64_t Q, int64_t ldp, int nq,
-                      int tiles_q, int64_t steps, int64_t units, int64_t ncl, float scale,
-                      int txn, float* __restrict__ Y, int64_t ldy) {
+    k_reduce_segments(const float* part, int64_t P, int64_t Q, int64_t ldp, int nq, int tiles_q,
+                      int64_t steps, int64_t units, int64_t ncl, float scale, int txn, float* Y,
+                      int64_t ldy) {
   using V = typename std::conditional<W == 4, float4, float>::type;
   constexpr int RU = 4;  // rows in flight per thread
   const int64_t total = P * ldp;
