@@ -17,6 +17,11 @@
 // main ones, and so is what they lose) and the main one is a chain of at most
 // 6 or 8 stages that is added, with IEEE adds, to the ones before it.  A
 // Rademacher S is exact in one BF16 value: s1 a1, then s1 a2 + s1 a3.
+// The parts of an element below 2^-110 reach into BF16's subnormals and lose
+// bits.  A column whose elements are all small in an item is therefore
+// multiplied by 2^48 on the way in and by 2^-48 on the way out (exact); which
+// columns these are is known when the item has been read, so such items run a
+// second time at the end.
 //
 // A CTA owns a 128 x NT tile of Y (NT <= 256: two accumulators of NT TMEM
 // columns) and a list of (tile, split of m) items:
@@ -74,8 +79,20 @@ constexpr uint32_t SLOT_MAX = OFF_A + 3 * NCH * A_CHUNK;
 constexpr uint32_t EPI_TILE = 32 * 16 * 4;
 constexpr uint32_t OFF_BAR = SLOTS * SLOT_MAX + N_EPI * EPI_TILE;
 constexpr uint32_t NUM_BARS = 2 * SLOTS + 3;
-constexpr uint32_t OFF_MISC = OFF_BAR + NUM_BARS * 8;  // abort flag, TMEM slot, chain flags
-constexpr uint32_t SMEM = OFF_MISC + 16 + 4 * 4 + 1024;  // + slack for 1 KB alignment
+constexpr uint32_t OFF_MISC = OFF_BAR + NUM_BARS * 8;  // abort flag, TMEM slot
+constexpr uint32_t OFF_SEEN = OFF_MISC + 16;           // column flags (Seen)
+constexpr int SEEN = 4;         // items whose flags are kept at a time
+constexpr int REDO_BITS = 512;  // items (modulo this) that run a second time
+struct Seen {
+  // columns 64 c + 2 l + x of an item's tile as bit l of word 2 c + x
+  uint32_t normal[SEEN][2 * NCH];  // an element of at least kSmall was seen
+  uint32_t small[SEEN][2 * NCH];   // a smaller one was, before any of those
+  uint32_t all[SEEN];              // normal elements were seen in every column
+  uint32_t redo[REDO_BITS / 32];   // items with columns that may be small all through,
+  uint32_t any_redo;               // and whether there are any
+  uint32_t scaled[2 * NCH];        // columns that the second run multiplies by kUp
+};
+constexpr uint32_t SMEM = OFF_SEEN + sizeof(Seen) + 1024;  // + slack for 1 KB alignment
 static_assert(SMEM <= 227 * 1024, "shared memory budget");
 static_assert(SLOT_MAX % 1024 == 0 && OFF_A % 1024 == 0, "swizzle atoms on 1 KB boundaries");
 static_assert(SLOTS * (SLOT_MAX - 3 * A_CHUNK) + N_EPI * 4 * EPI_TILE <= OFF_BAR, "staging tiles");
@@ -83,11 +100,12 @@ static_assert(GROUPS <= SLOTS, "worker groups vs ring depth");
 
 // |a| above this rounds to an infinite BF16; such a value is truncated.
 constexpr float kRoundsToInf = 0x1.fep127f;
-// Magnitudes from 2^-110 on split without error; an item's tile of A whose
-// largest magnitude is below this is multiplied in FP32 FMAs instead.
-constexpr float kTiny = 0x1p-100f;
-// What the workers saw in an item's rows of A.
-constexpr int kSawTiny = 1, kSawNormal = 2;
+// Magnitudes from 2^-110 on split without error.  A column of an item with
+// none of at least kSmall runs again, times kUp: its elements are then below
+// 2^-52 and the smallest subnormal at 2^-101.  (In a column with one, what the
+// others lose is below 2^-33 of it.)
+constexpr float kSmall = 0x1p-100f;
+constexpr float kUp = 0x1p48f, kDown = 0x1p-48f;
 
 struct F32Params {
   const float* A;
@@ -153,41 +171,88 @@ __device__ __forceinline__ void split3(float2 x, uint32_t (&w)[3]) {
   w[2] = pack_bf16(q.x, q.y);
 }
 
-// A row of an item's tile in FP32 FMAs, for a tile of A too small in
-// magnitude to split (rare: all of it below 2^-100), W columns per generated
-// entry.
-__device__ __noinline__ void slow_item(const F32Params& p, int64_t row, int64_t q0, int64_t q1,
-                                       int64_t l0, int64_t l1, float* out) {
-  constexpr int W = 16;
-  const PhiloxKey key{p.rk.k[0], p.rk.k[1]};
-  for (int64_t c = q0; c < q1; c += W) {
-    float acc[W];
+// The columns of an item (`rows` rows of its tile of A) that hold small
+// elements and no others, as bits of seen->scaled; whether there are any.  By
+// all threads of the block, with the ring idle.
+__device__ __noinline__ bool find_small_columns(const float* A, int64_t lda, int64_t rows,
+                                                int ncols, Seen* seen, uint32_t* colmax) {
+  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
+  for (int c = tid; c < 64 * NCH; c += THREADS) colmax[c] = 0u;
+  if (tid < 2 * NCH) seen->scaled[tid] = 0u;
+  __syncthreads();
+  for (int c = lane; c < ncols; c += 32) {
+    uint32_t mx = 0u;  // magnitudes order as their bits do (NaN above all)
+#pragma unroll 4
+    for (int64_t l = warp; l < rows; l += THREADS / 32)
+      mx = max(mx, __float_as_uint(A[l * lda + c]) & 0x7fffffffu);
+    atomicMax(colmax + c, mx);
+  }
+  __syncthreads();
+  bool any = false;
+  if (tid < ncols && colmax[tid] != 0u && colmax[tid] < __float_as_uint(kSmall)) {
+    any = true;
+    atomicOr(seen->scaled + 2 * (tid >> 6) + (tid & 1), 1u << ((tid & 63) >> 1));
+  }
+  return __syncthreads_or(any) != 0;
+}
+
+// What a warp has to find out about the columns of an item: nothing (any more),
+// whether any holds small elements, or first whether all of them are normal.
+constexpr int kLookNone = 0, kLookSmall = 1, kLookFirst = 2;
+
+// Two rows of an item show these magnitudes (the larger of the two) in this
+// lane's columns; the flags of column i = 2 c + x are bits i (a normal element)
+// and 8 + i (any but zeros) of `cols`.  Dense data of ordinary size is done
+// with after the first rows; without small elements the others cost a
+// comparison.
+__device__ __forceinline__ int look_at_columns(const float2 (&mx)[NCH], int nconv, int look,
+                                               uint32_t* cols, uint32_t* all) {
+  if (look == kLookFirst) {
+    float least = kSmall;
 #pragma unroll
-    for (int j = 0; j < W; ++j) acc[j] = 0.0f;
-    const int nc = static_cast<int>(min(static_cast<int64_t>(W), q1 - c));
-    for (int64_t l = l0; l < l1; l += 4) {
-      const float4 g = gen4(p.dist, key, static_cast<uint32_t>(row), static_cast<uint32_t>(l));
-      const int nl = static_cast<int>(min(static_cast<int64_t>(4), l1 - l));
-      for (int i = 0; i < nl; ++i) {
-        const float gi = i == 0 ? g.x : i == 1 ? g.y : i == 2 ? g.z : g.w;
-        const float* a = p.A + (l + i) * p.lda + c;
-#pragma unroll
-        for (int j = 0; j < W; ++j)
-          if (j < nc) acc[j] = __fmaf_rn(gi, a[j], acc[j]);
-      }
+    for (int c = 0; c < NCH; ++c)
+      if (c < nconv) least = fminf(least, fminf(mx[c].x, mx[c].y));
+    if (__all_sync(0xffffffffu, least >= kSmall)) {
+      *all = 1u;
+      return kLookNone;
     }
+  }
+  uint32_t low = 0xffffffffu;  // zeros wrap around to the largest number
 #pragma unroll
-    for (int j = 0; j < W; ++j)
-      if (j < nc) out[c + j] = acc[j];
+  for (int c = 0; c < NCH; ++c)
+    low = min(low, min(__float_as_uint(mx[c].x) - 1u, __float_as_uint(mx[c].y) - 1u));
+  if (__any_sync(0xffffffffu, low < __float_as_uint(kSmall) - 1u)) {
+#pragma unroll
+    for (int i = 0; i < 2 * NCH; ++i) {
+      const float m = i & 1 ? mx[i >> 1].y : mx[i >> 1].x;
+      if (m >= kSmall) *cols |= 1u << i;
+      if (m > 0.0f) *cols |= 0x100u << i;
+    }
+  }
+  return kLookSmall;
+}
+
+// A warp's flags of an item, for the epilogue.
+__device__ __noinline__ void publish_columns(uint32_t cols, uint32_t* normal, uint32_t* small) {
+  for (int i = 0; i < 2 * NCH; ++i) {
+    const uint32_t n = __ballot_sync(0xffffffffu, (cols >> i) & 1u);
+    const uint32_t z = __ballot_sync(0xffffffffu, (cols >> (8 + i)) & 1u) & ~n;
+    if ((threadIdx.x & 31) == 0) {
+      if (n) atomicOr(normal + i, n);
+      if (z) atomicOr(small + i, z);
+    }
   }
 }
 
-template <int DIST>
-__global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_constant__ CUtensorMap pmap, const F32Params p) {
+// The roles of a block's warps over its items first_item, + item_step, ... below
+// end_item, after `runs` calls and in them g stages, gc chains and j items.
+// AGAIN: items with columns to scale.
+template <int DIST, bool AGAIN>
+__device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Params& p,
+                                          uint8_t* smem, uint32_t tmem, int first_item,
+                                          int item_step, int end_item, uint32_t runs, int g,
+                                          int gc, int j) {
   constexpr int NS = DIST == kRademacher ? 1 : 3;  // parts of S
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~static_cast<uintptr_t>(1023));
   const uint32_t sbase = smem_u32(smem);
   const uint32_t bar0 = sbase + OFF_BAR;
   // full: a worker group has written the slot; empty: its MMAs have completed
@@ -196,40 +261,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
   const uint32_t acc_full = bar0 + 8u * (2 * SLOTS);
   const uint32_t acc_empty = acc_full + 8u;
   const uint32_t drain_bar = acc_full + 16u;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_MISC);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_MISC + 4);
-  // kSawTiny / kSawNormal of the last four items: the workers are at most
-  // three stages, hence three items, ahead of the epilogue
-  int* saw = reinterpret_cast<int*>(smem + OFF_MISC + 16);
+  // flags of the last four items: the workers are at most three stages, hence
+  // three items, ahead of the epilogue
+  Seen* seen = reinterpret_cast<Seen*>(smem + OFF_SEEN);
+  const Abort ab{reinterpret_cast<volatile int*>(smem + OFF_MISC), p.status, p.timeout_ns};
   const int warp = uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < SLOTS; ++i) {
-      mbar_init(full(i), GROUP_WARPS);
-      mbar_init(empty(i), 1);
-    }
-    mbar_init(acc_full, 1);
-    mbar_init(acc_empty, N_EPI);
-    mbar_init(drain_bar, 1);
-    *abort_flag = 0;
-    for (int i = 0; i < 4; ++i) saw[i] = 0;
-    mbar_fence_init();
-  }
-  if (warp == 0) {
-    tmem_alloc(smem_u32(tmem_slot), 512u);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  pdl_wait();
-  pdl_trigger();
-  const uint32_t tmem = uniform(*tmem_slot);
-  const Abort ab{abort_flag, p.status, p.timeout_ns};
   const uint32_t a_part = static_cast<uint32_t>(p.nt / 64) * A_CHUNK;  // one part of A in a slot
   const uint32_t slot_bytes = OFF_A + 3u * a_part;
-  const int first_item = static_cast<int>(blockIdx.x), item_step = static_cast<int>(gridDim.x);
 
   if (warp == 0) {  // the whole warp; one lane issues
     const uint32_t el = elect_one();
@@ -237,9 +276,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
         idesc_bf16_f32(BM, static_cast<uint32_t>(p.nt)) | (1u << 16);  // B is MN-major
     const uint64_t a_base = smem_desc(sbase, 128u, 256u);
     const uint64_t b_base = smem_desc_sw128(sbase + OFF_A, A_CHUNK, 1024u);
-    int g = 0, gc = 0, j = 0;
     bool stop = false;
-    for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+    for (int idx = first_item; idx < end_item && !stop; idx += item_step, ++j) {
       const int nsteps = get_item(p, idx).nsteps;
       int in_chain = 0;
       for (int s = 0; s < nsteps; ++s, ++g) {
@@ -250,7 +288,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
             stop = true;
             break;
           }
-          if (s == 0 && lane == 0) saw[(j - 1) & 3] = 0;
+          if (s == 0) {
+            const int e = (j - 1) % SEEN;
+            if (lane < 2 * NCH) seen->normal[e][lane] = seen->small[e][lane] = 0u;
+            if (lane == 0) seen->all[e] = 0u;
+          }
           __syncwarp();
         }
         if (!mbar_wait_warp(full(so), (g / SLOTS) & 1, ab, 0x22, g)) {
@@ -285,7 +327,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
       }
     }
     mma_commit(drain_bar, el);
-    drain_wait(drain_bar, 0, 200000000ull);
+    drain_wait(drain_bar, runs & 1, 200000000ull);
   } else if (warp < W_WORK0) {
     // ---- epilogue: lanes are accumulator rows, main in columns 0 .. nt - 1,
     // cross in 256 .. ----
@@ -293,11 +335,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
     const int ntile = p.nt == 64 * NCH ? 1 : 4;
     uint8_t* tiles = smem + SLOTS * slot_bytes + (warp - W_EPI0) * ntile * EPI_TILE;
     const uint32_t usw = (static_cast<uint32_t>(lane) >> 1) & 3u;
-    int gc = 0, j = 0;
     bool stop = false;
-    for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+    for (int idx = first_item; idx < end_item && !stop; idx += item_step, ++j) {
       const Item it = get_item(p, idx);
-      float* part = p.part + static_cast<int64_t>(it.z) * p.P * p.ldp;
       const int64_t r0 = it.p0 + quarter * 32;
       for (int c0 = 0; c0 < it.nchains; ++c0, ++gc) {
         const bool ok = mbar_wait(acc_full, gc & 1, ab, 0x34, gc);
@@ -311,13 +351,17 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
         // stay in chain order
         if (lane == 0) bulk_wait<0>();
         __syncwarp();
-        const bool slow = last && *static_cast<volatile int*>(saw + (j & 3)) == kSawTiny;
-        const int nchunk = r0 >= p.P || slow
-                               ? 0
-                               : static_cast<int>((min(static_cast<int64_t>(p.nt), p.Q - it.q0) + 31) / 32);
-        if (slow && r0 + lane < p.P)
-          slow_item(p, r0 + lane, it.q0, min(p.Q, it.q0 + p.nt), it.lbeg, it.lend,
-                    part + (r0 + lane) * p.ldp);
+        if (last && !AGAIN && warp == W_EPI0 && lane < 2 * NCH) {
+          const volatile Seen* f = seen;
+          const int e = j % SEEN;
+          if (f->all[e] == 0u && (f->small[e][lane] & ~f->normal[e][lane]) != 0u) {
+            atomicOr(seen->redo + (j % REDO_BITS) / 32, 1u << (j % 32));
+            seen->any_redo = 1u;
+          }
+        }
+        const int nchunk =
+            r0 >= p.P ? 0
+                      : static_cast<int>((min(static_cast<int64_t>(p.nt), p.Q - it.q0) + 31) / 32);
         int nb = 0;
         for (int ci = 0; ci < nchunk; ++ci) {
           uint32_t v[32], w[32];
@@ -337,6 +381,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
             }
           } else {
             tmem_ld_wait();
+          }
+          if constexpr (AGAIN) {  // columns that were multiplied by kUp
+            const uint32_t* m = seen->scaled + (ci >> 1) * 2;
+            const uint32_t even = m[0] >> (16 * (ci & 1)), odd = m[1] >> (16 * (ci & 1));
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (((i & 1 ? odd : even) >> (i >> 1)) & 1u)
+                v[i] = __float_as_uint(__fmul_rn(__uint_as_float(v[i]), kDown));
           }
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
@@ -364,10 +416,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
             __syncwarp();
             if (lane == 0) {
               if (first)
-                tma_store_3d(&pmap, smem_u32(tile), static_cast<int32_t>(col),
+                tma_store_3d(pmap, smem_u32(tile), static_cast<int32_t>(col),
                              static_cast<int32_t>(r0), it.z);
               else
-                tma_reduce_add_3d(&pmap, smem_u32(tile), static_cast<int32_t>(col),
+                tma_reduce_add_3d(pmap, smem_u32(tile), static_cast<int32_t>(col),
                                   static_cast<int32_t>(r0), it.z);
               bulk_commit();
             }
@@ -389,11 +441,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
     const uint32_t rbase = static_cast<uint32_t>(w * 8 + (lane & 7));
     const uint32_t s_off =
         (rbase & 7u) * 16u + (rbase >> 3) * 256u + (qd >> 1) * 128u + (qd & 1u) * 8u;
-    int g = 0, j = 0;
     bool stop = false;
-    for (int idx = first_item; idx < p.nitems && !stop; idx += item_step, ++j) {
+    for (int idx = first_item; idx < end_item && !stop; idx += item_step, ++j) {
       const Item it = get_item(p, idx);
       const int g_item = g;
+      int look = AGAIN ? kLookNone : kLookFirst;
+      uint32_t cols = 0u;
       // columns of the tile: nfull whole chunks, then perhaps part of one,
       // where lanes past the last column read that one again (what they
       // contribute to is never read out)
@@ -407,8 +460,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
         uint8_t* slot = smem + static_cast<uint32_t>(so) * slot_bytes;
         const int64_t cbase = it.lbeg + static_cast<int64_t>(s) * SL;
         bool ok = true;
-        float amax = 0.0f;
-        float hmax = 0.0f;
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
           // this warp's rows 16 half + 2 w, + 1 of the stage, columns 2 lane,
@@ -474,13 +525,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
               }
             }
           }
-          hmax = 0.0f;
+          if constexpr (AGAIN) {
 #pragma unroll
-          for (int j2 = 0; j2 < 2; ++j2)
+            for (int c = 0; c < NCH; ++c) {
+              const float2 up = f2((seen->scaled[2 * c] >> lane) & 1u ? kUp : 1.0f,
+                                   (seen->scaled[2 * c + 1] >> lane) & 1u ? kUp : 1.0f);
 #pragma unroll
-            for (int c = 0; c < NCH; ++c)
-              hmax = fmaxf(hmax, fmaxf(fabsf(x[j2][c].x), fabsf(x[j2][c].y)));
-          amax = fmaxf(amax, hmax);
+              for (int j2 = 0; j2 < 2; ++j2) x[j2][c] = __fmul2_rn(x[j2][c], up);
+            }
+          }
+          float2 mx[NCH];
+          float hmax = 0.0f;
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) {
+            mx[c] = f2(fmaxf(fabsf(x[0][c].x), fabsf(x[1][c].x)),
+                       fmaxf(fabsf(x[0][c].y), fabsf(x[1][c].y)));
+            hmax = fmaxf(hmax, fmaxf(mx[c].x, mx[c].y));
+          }
+          if (look != kLookNone)
+            look = look_at_columns(mx, nconv, look, &cols, seen->all + j % SEEN);
           auto store = [&](auto huge) {
 #pragma unroll
             for (int j2 = 0; j2 < 2; ++j2) {
@@ -507,23 +570,102 @@ __global__ void __launch_bounds__(THREADS, 1) k_sketch_fp32_left(const __grid_co
           stop = true;
           break;
         }
-        const bool normal = __any_sync(0xffffffffu, amax >= kTiny);
-        const bool tiny = __any_sync(0xffffffffu, amax > 0.0f);
+        // (the group's last stage of the item)
+        if (s + GROUPS >= it.nsteps && __any_sync(0xffffffffu, cols != 0u))
+          publish_columns(cols, seen->normal[j % SEEN], seen->small[j % SEEN]);
         fence_proxy_async_smem();  // the slot is read by the tensor core
         __syncwarp();
-        if (lane == 0) {
-          if (tiny) atomicOr(saw + (j & 3), normal ? kSawNormal : kSawTiny);
-          mbar_arrive(full(so));
-        }
+        if (lane == 0) mbar_arrive(full(so));
       }
       g = g_item + it.nsteps;
     }
   }
+}
 
+// The second run: items with columns of small elements, one by one, after the
+// first one and a __syncthreads().  A sketch whose items all have such columns
+// takes almost three times as long (30011 x 333, k = 666 192 -> 525 us; the
+// CUDA cores take 644).  That its code is there at all costs the first run
+// registers, inlined or not (192 us against 174 without it, 4096 x 256, k = 64
+// 14.4 against 12.7), about what the code it stands for, FP32 FMAs in the
+// epilogue warps, cost before (194 and 14.0 us; 13.3 ms for small elements).
+template <int DIST>
+__device__ __noinline__ void run_again(const CUtensorMap* pmap, const F32Params& p, uint8_t* smem,
+                                       uint32_t tmem) {
+  Seen* seen = reinterpret_cast<Seen*>(smem + OFF_SEEN);
+  const volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_MISC);
+  const int item_step = static_cast<int>(gridDim.x);
+  int g = 0, gc = 0, j = 0;  // the first run's
+  for (int idx = static_cast<int>(blockIdx.x); idx < p.nitems; idx += item_step, ++j) {
+    const Item it = get_item(p, idx);
+    g += it.nsteps;
+    gc += it.nchains;
+  }
+  uint32_t runs = 1;
+  int jj = 0;  // number of the item among the block's
+  for (int idx = static_cast<int>(blockIdx.x); idx < p.nitems && *abort_flag == 0;
+       idx += item_step, ++jj) {
+    if (((seen->redo[(jj % REDO_BITS) / 32] >> (jj % 32)) & 1u) == 0u) continue;
+    const Item it = get_item(p, idx);
+    if (!find_small_columns(p.A + it.lbeg * p.lda + it.q0, p.lda, it.lend - it.lbeg,
+                            static_cast<int>(min(static_cast<int64_t>(p.nt), p.Q - it.q0)), seen,
+                            reinterpret_cast<uint32_t*>(smem)))
+      continue;
+    run_items<DIST, true>(pmap, p, smem, tmem, idx, item_step, idx + 1, runs++, g, gc, j);
+    g += it.nsteps;
+    gc += it.nchains;
+    ++j;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  }
+}
+
+template <int DIST>
+__global__ void __launch_bounds__(THREADS, 1)
+    k_sketch_fp32_left(const __grid_constant__ CUtensorMap pmap,
+                       const __grid_constant__ F32Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_MISC);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_MISC + 4);
+  Seen* seen = reinterpret_cast<Seen*>(smem + OFF_SEEN);
+  const int warp = uniform(static_cast<int>(threadIdx.x >> 5));
+
+  if (threadIdx.x == 0) {
+    const uint32_t bar0 = smem_u32(smem) + OFF_BAR;  // (see run_items)
+    for (int i = 0; i < SLOTS; ++i) {
+      mbar_init(bar0 + 8u * i, GROUP_WARPS);
+      mbar_init(bar0 + 8u * (SLOTS + i), 1);
+    }
+    mbar_init(bar0 + 8u * (2 * SLOTS), 1);
+    mbar_init(bar0 + 8u * (2 * SLOTS + 1), N_EPI);
+    mbar_init(bar0 + 8u * (2 * SLOTS + 2), 1);
+    *abort_flag = 0;
+    mbar_fence_init();
+  }
+  for (uint32_t i = threadIdx.x; i < sizeof(Seen) / 4; i += THREADS)
+    reinterpret_cast<uint32_t*>(seen)[i] = 0u;
+  if (warp == 0) {
+    tmem_alloc(smem_u32(tmem_slot), 512u);
+    tmem_relinquish();
+  }
   tc_fence_before();
   __syncthreads();
+  tc_fence_after();
+  pdl_wait();
+  pdl_trigger();
+  const uint32_t tmem = uniform(*tmem_slot);
+
+  run_items<DIST, false>(&pmap, p, smem, tmem, static_cast<int>(blockIdx.x),
+                         static_cast<int>(gridDim.x), p.nitems, 0u, 0, 0, 0);
+  // every chain has been read out (or the block gives up)
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (__builtin_expect(seen->any_redo != 0u, 0)) run_again<DIST>(&pmap, p, smem, tmem);
   if (warp == 0) {
-    tc_fence_after();
     __syncwarp();
     tmem_dealloc(tmem, 512u);
   }
