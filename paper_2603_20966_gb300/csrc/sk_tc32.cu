@@ -14,8 +14,9 @@
 // each exact in the tensor core, summed in FP32.  The tensor core truncates
 // where an FMA rounds, which shrinks a sum by about 2^-26 per K step, so the
 // two groups have accumulators of their own (the cross terms are 2^-8 of the
-// main ones, and so is what they lose) and the main one is a chain of at most
-// 6 or 8 stages that is added, with IEEE adds, to the ones before it.  A
+// main ones, and so is what they lose): the main one is a chain of at most
+// 6 or 8 stages that is added, with IEEE adds, to the ones before it, the
+// cross one is added with every chain that ends 128 stages or so.  A
 // Rademacher S is exact in one BF16 value: s1 a1, then s1 a2 + s1 a3.
 // The parts of an element below 2^-110 reach into BF16's subnormals and lose
 // bits.  A column whose elements are all small in an item is therefore
@@ -59,6 +60,13 @@ constexpr int NCH = 4;       // most 64-column chunks of a tile
 // Most stages per chain of the main accumulator: 192 rows of m (Rademacher
 // products are BF16 values and truncate less: 1024).
 constexpr int CHAIN = 6, CHAIN_LONG = 8, CHAIN_R = 32;
+// Stages after which the cross accumulator is read out with the chain that
+// ends there and starts again.  What it loses grows with its length: never
+// read out before an item's end, one split of 2^18, 2^20 and 2^22 rows had
+// errors of 3.6e-6, 1.4e-5 and 5.7e-5 (Gaussian S; the CUDA cores 6.5e-6,
+// 1.3e-5 and 2.6e-5), with this 6.2e-7, 1.2e-6 and 2.3e-6.  32 and 64 stages
+// have the same errors and cost up to 1 %, 128 cost 0.2 %.
+constexpr int CROSS = 128;
 constexpr int64_t kLongRows = 16384;  // rows of m from which chains are CHAIN_LONG
 constexpr int N_EPI = 4;
 constexpr int GROUPS = 2, GROUP_WARPS = 8;
@@ -116,6 +124,7 @@ struct F32Params {
   int tiles_p, tiles_q, nitems;
   int nt;     // columns per tile, a multiple of 64
   int chain;  // stages per accumulation chain
+  int cross;  // chains per accumulation of the cross terms
   int vec2;   // rows of A on 8-byte boundaries
   int dist;
   PhiloxRoundKeys rk;
@@ -279,7 +288,7 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
     bool stop = false;
     for (int idx = first_item; idx < end_item && !stop; idx += item_step, ++j) {
       const int nsteps = get_item(p, idx).nsteps;
-      int in_chain = 0;
+      int in_chain = 0, in_cross = 0;  // stages of the chain, chains of the cross terms so far
       for (int s = 0; s < nsteps; ++s, ++g) {
         const int so = g % SLOTS;
         if (in_chain == 0 && gc > 0) {
@@ -310,7 +319,7 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
                      b0 + ((static_cast<uint32_t>(ap) * a_part + ks * 2048u) >> 4), idesc, acc, el);
           };
           mma(0, 0, 0u, in_chain > 0 || ks > 0 ? 1u : 0u);
-          mma(0, 1, 256u, s > 0 || ks > 0 ? 1u : 0u);
+          mma(0, 1, 256u, in_chain > 0 || in_cross > 0 || ks > 0 ? 1u : 0u);
           mma(0, 2, 256u, 1u);
           if (NS == 3) {
             mma(1, 0, 256u, 1u);
@@ -322,6 +331,7 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
         if (++in_chain == p.chain || s == nsteps - 1) {
           mma_commit(acc_full, el);
           in_chain = 0;
+          if (++in_cross == p.cross) in_cross = 0;
           ++gc;
         }
       }
@@ -339,6 +349,7 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
     for (int idx = first_item; idx < end_item && !stop; idx += item_step, ++j) {
       const Item it = get_item(p, idx);
       const int64_t r0 = it.p0 + quarter * 32;
+      int in_cross = 0;
       for (int c0 = 0; c0 < it.nchains; ++c0, ++gc) {
         const bool ok = mbar_wait(acc_full, gc & 1, ab, 0x34, gc);
         if (!__all_sync(0xffffffffu, ok)) {
@@ -347,6 +358,8 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
         }
         tc_fence_after();
         const bool first = c0 == 0, last = c0 == it.nchains - 1;
+        const bool with_cross = last || ++in_cross == p.cross;
+        if (with_cross) in_cross = 0;
         // the earlier chains' adds have been performed: those of one element
         // stay in chain order
         if (lane == 0) bulk_wait<0>();
@@ -368,7 +381,7 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
           const uint32_t src =
               tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(ci * 32);
           tmem_ld32(src, v);
-          if (last) {
+          if (with_cross) {
             tmem_ld32(src + 256u, w);
             tmem_ld_wait();
 #pragma unroll
@@ -684,7 +697,7 @@ int sm_count() {
 }
 
 struct F32Plan {
-  int nt, splits, chain;
+  int nt, splits, chain, cross;
   int64_t tiles_p, tiles_q, chunk, ldp;
 };
 
@@ -714,6 +727,7 @@ F32Plan plan_f32(const GemmShape& s, int dist = kGaussian) {
   const int64_t cap = dist == kRademacher ? CHAIN_R : s.L >= kLongRows ? CHAIN_LONG : CHAIN;
   const int64_t nchains = (per + cap - 1) / cap;
   pl.chain = static_cast<int>((per + nchains - 1) / nchains);
+  pl.cross = std::max(1, CROSS / pl.chain);
   return pl;
 }
 
@@ -761,6 +775,9 @@ cudaError_t launch_f32(const CUtensorMap& pmap, const F32Params& p, unsigned gri
 //   64 x 32, 64          21 -> 13 us      1.5e-7 -> 6.7e-8
 //   32 x 512, 512        15.2 -> 17.5 us  (one stage: stays on the CUDA cores)
 // Chains of 11, 19 and 32 stages had errors of 3.4e-7, 5.8e-7 and 8.3e-7.
+// Sums that all grow the same way lose most to truncation: a uniform S and an
+// A without negative elements have 3.4e-7 at 30011 x 333, k = 666 (the CUDA
+// cores 1.2e-7, a normal A 2.3e-7 here and 5.2e-7 there).
 size_t tc32_workspace_bytes(const GemmShape& s) {
   if (!s.left || s.L < 2 * SL) return 0;
   // (a k of more than 65535 tiles is refused, as the CUDA-core form does)
@@ -794,6 +811,7 @@ cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float
   p.nitems = static_cast<int>(pl.tiles_p * pl.tiles_q * pl.splits);
   p.nt = pl.nt;
   p.chain = pl.chain;
+  p.cross = pl.cross;
   p.vec2 = reinterpret_cast<uintptr_t>(A) % 8 == 0 && lda % 2 == 0;
   p.dist = h->dist;
   p.rk = round_keys(make_key(h->seed));
