@@ -234,7 +234,9 @@ sk_status sk_materialize(sk_handle h, int64_t row0, int64_t col0, int64_t rows, 
  * SK_FP32 left sketches run on the tensor cores where the buffer holds their
  * partials, which the size above does; a smaller one is taken as long as it
  * holds the partials of the CUDA cores' form, which then runs (also in a
- * server whose budget holds no more, and in sk_apply_left_noalloc). */
+ * server whose budget holds no more, in sk_apply_left_noalloc, and where
+ * handle-owned scratch cannot grow: in a stream capture, or when the device
+ * has no memory left). */
 sk_status sk_workspace_size(sk_handle h, int side, int64_t m, int64_t n, size_t* bytes);
 sk_status sk_set_workspace(sk_handle h, void* ptr, size_t bytes);
 

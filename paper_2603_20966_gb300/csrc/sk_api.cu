@@ -38,7 +38,7 @@ sk_status from_cuda(cudaError_t e) { return sk::status_from_cuda(e); }
 bool valid_dist(int d) { return d == SK_GAUSSIAN || d == SK_RADEMACHER || d == SK_UNIFORM; }
 bool valid_prec(int p) { return p == SK_FP32 || p == SK_BF16X2 || p == SK_FP8E4M3; }
 
-// least: what a lent buffer has to hold (the tensor-core forms use some more
+// least: what a sketch cannot do without (the tensor-core forms use some more
 // where they can)
 size_t workspace_for(const sk_sketch* h, const GemmShape& s, bool least = false) {
   if (h->prec == SK_FP32) {
@@ -70,10 +70,26 @@ sk_status ensure_workspace(sk_sketch* h, size_t need) {
   return SK_OK;
 }
 
-// The scratch of an apply call; a lent buffer has to hold only the least.
-sk_status ensure_workspace(sk_sketch* h, const GemmShape& s) {
+// Whether memory must not be allocated or freed now: `st` is being captured
+// (or is the legacy stream while another one is).
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &c) == cudaSuccess) return c != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// The scratch of an apply call.  A lent buffer has to hold only the least, and
+// so has scratch of the handle's that cannot grow: under capture, or where
+// the memory for more cannot be had.
+sk_status ensure_workspace(sk_sketch* h, const GemmShape& s, cudaStream_t st) {
   const bool lent = !h->ws_owned && h->ws != nullptr;
-  return ensure_workspace(h, workspace_for(h, s, lent));
+  const size_t need = workspace_for(h, s, lent);
+  if (lent || h->ws_bytes >= need) return ensure_workspace(h, need);
+  const size_t least = workspace_for(h, s, true);
+  if (h->ws_bytes >= least && capturing(st)) return SK_OK;
+  const sk_status r = ensure_workspace(h, need);
+  return r == SK_ENOMEM && least < need ? ensure_workspace(h, least) : r;
 }
 
 sk_status check_apply(const sk_sketch* h, const float* A, int64_t m, int64_t n, int64_t lda,
@@ -106,9 +122,9 @@ sk_status apply(sk_sketch* h, const float* A, int64_t m, int64_t n, int64_t lda,
   }
   if (h->prec == SK_FP8E4M3 && ((reinterpret_cast<uintptr_t>(Y) & 15u) || ldy % 4 != 0))
     return SK_EINVAL;
-  st = ensure_workspace(h, s);
-  if (st != SK_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  st = ensure_workspace(h, s, cs);
+  if (st != SK_OK) return st;
   cudaError_t e;
   if (h->prec == SK_FP32)
     e = sk::fp32_sketch(h, s, A, lda, Y, ldy, h->ws, h->ws_bytes, cs);
@@ -270,7 +286,7 @@ sk_status sk_apply_left_stored(sk_handle h, const void* S, int64_t lds, const fl
   s.L = m;
   st = sk::tc_check(s, A, lda, Y, ldy);
   if (st != SK_OK) return st;
-  st = ensure_workspace(h, s);
+  st = ensure_workspace(h, s, static_cast<cudaStream_t>(stream));
   if (st != SK_OK) return st;
   return from_cuda(sk::tc_sketch_left_stored(h, s, S, lds, A, lda, Y, ldy, h->ws, h->ws_bytes,
                                              static_cast<cudaStream_t>(stream)));
