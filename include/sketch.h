@@ -437,9 +437,9 @@ sk_status sk_debug_status(sk_handle h, void* stream, int32_t out[4]);
  * core launches, at least 1 ms; 0 restores the default of 2 s.
  * stall_stage >= 0: in later BF16 left sketches on this handle the TMA
  * producer issues no copy for that pipeline stage (stages counted from 0
- * over each CTA's, or CTA pair's, run of a launch), so every wait that
- * depends on it gives up after
- * limit_ns: the kernel records SK_ETIMEOUT and the waiting site (see
+ * over each CTA's, or CTA pair's, run of a launch), and in FP32 left ones on
+ * the tensor cores the workers never hand it on, so every wait that depends
+ * on it gives up after limit_ns: the kernel records SK_ETIMEOUT and the waiting site (see
  * sk_debug_status), waits (again bounded) for the copies and MMAs already
  * in flight, frees its tensor memory and exits; Y is then undefined.
  * stall_stage < 0 turns the injection off.  Errors: SK_EINVAL. */

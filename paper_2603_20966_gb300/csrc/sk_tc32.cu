@@ -130,6 +130,9 @@ struct F32Params {
   PhiloxRoundKeys rk;
   int* status;
   uint64_t timeout_ns;
+  // failure-injection hook of the tests, -1 otherwise: this stage (counted over
+  // a block's items) is never handed to the MMA issuer
+  int64_t stall_stage;
 };
 
 struct Item {
@@ -588,7 +591,7 @@ __device__ __forceinline__ void run_items(const CUtensorMap* pmap, const F32Para
           publish_columns(cols, seen->normal[j % SEEN], seen->small[j % SEEN]);
         fence_proxy_async_smem();  // the slot is read by the tensor core
         __syncwarp();
-        if (lane == 0) mbar_arrive(full(so));
+        if (lane == 0 && g != p.stall_stage) mbar_arrive(full(so));
       }
       g = g_item + it.nsteps;
     }
@@ -817,6 +820,7 @@ cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float
   p.rk = round_keys(make_key(h->seed));
   p.status = h->d_status;
   p.timeout_ns = h->wait_limit_ns;
+  p.stall_stage = h->stall_stage;
   CUtensorMap pmap;
   if (!encode_partials(&pmap, p.part, s.Q, s.P, pl.splits, pl.ldp)) return cudaErrorInvalidValue;
   const unsigned grid = static_cast<unsigned>(std::min(p.nitems, sm_count()));
