@@ -12,10 +12,17 @@ import torch
 from . import _native as N
 
 
+# torch's current raw stream without a Stream object, which costs more than a
+# small sketch's launches (torch's inductor calls the same function); None in a
+# torch that has no such function
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_of(A: torch.Tensor) -> int:
-    """torch's current stream on A's device, as the library takes it: without
-    a Stream object, which costs more than a small sketch's launches."""
-    return torch._C._cuda_getCurrentRawStream(A.get_device())
+    """torch's current stream on A's device, as the library takes it."""
+    if _raw_stream is None:
+        return torch.cuda.current_stream(A.device).cuda_stream
+    return _raw_stream(A.get_device())
 
 
 class Sketch:
