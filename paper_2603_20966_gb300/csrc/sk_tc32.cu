@@ -57,8 +57,15 @@ constexpr int BM = 128;      // rows of S per tile
 constexpr int SL = 32;       // rows of m per stage
 constexpr int SLOTS = 3;     // stages in the ring
 constexpr int NCH = 4;       // most 64-column chunks of a tile
-// Most stages per chain of the main accumulator: 192 rows of m (Rademacher
-// products are BF16 values and truncate less: 1024).
+// Most stages per chain of the main accumulator: 192 rows of m, 256 from
+// kLongRows on (Rademacher products are BF16 values and truncate less: 1024).
+// Longer chains are faster and truncate more; these stay at half the error of
+// the CUDA cores' form.  With chains of 4, 6, 8, 10 stages and there (Gaussian
+// S, n = 512, k = 2048):
+//   4096 rows    1.4, 1.7, 1.7, 3.0e-7, there 3.3e-7    126, 107, 107, 93 us
+//   8192 rows    1.5, 1.6, 2.1, 2.8e-7, there 4.6e-7    208, 190, 175, 163 us
+//   16384 rows   1.5, 2.0, 2.4, 2.9e-7, there 6.4e-7    396, 353, 318, 303 us
+//   65536 rows   1.9, 2.2, 2.6, 3.1e-7, there 12.6e-7   1.45, 1.29, 1.20, 1.14 ms
 constexpr int CHAIN = 6, CHAIN_LONG = 8, CHAIN_R = 32;
 // Stages after which the cross accumulator is read out with the chain that
 // ends there and starts again.  What it loses grows with its length: never
@@ -712,7 +719,7 @@ F32Plan plan_f32(const GemmShape& s, int dist = kGaussian) {
   pl.ldp = (s.Q + 3) / 4 * 4;
   // splits of m that fill whole waves of CTAs, each at least one stage per
   // worker group; where the most of them leave SMs idle, narrower tiles (each
-  // generates its S again, but drains sooner: 4096 x 256, k = 64 18.7 -> 16.4
+  // generates its S again, but drains sooner: 4096 x 256, k = 64 18.5 -> 15.4
   // us); more than 64 splits (whose partials the reduction reads) only of
   // eight stages or more (65536 x 32, k = 64 57 -> 31 us)
   const int64_t sms = sm_count();

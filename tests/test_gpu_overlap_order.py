@@ -55,3 +55,54 @@ def test_every_call_of_a_graph_sees_its_own_data(side, form, dist, k, m, n):
             for i, y in enumerate(ys):
                 assert torch.equal(y, want[i % 4]), i
         assert sk.status() == 0
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("side,form,k,m,n", [("left", 0, 64, 60000, 256), ("left", 1, 64, 60000, 256),
+                                             ("right", 1, 100, 9000, 3000)])
+def test_inputs_written_on_another_stream(side, form, k, m, n, captured):
+    """A written on a second stream that the sketch's stream has waited for,
+    and Y read there afterwards."""
+    require_gpu()
+    import paper_2603_20966_gb300 as P
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    src = [torch.randn(m, n, device="cuda", generator=gen) for _ in range(3)]
+    A = torch.empty(m, n, device="cuda")
+    shape = (k, n) if side == "left" else (m, k)
+    ys = [torch.empty(shape, device="cuda") for _ in src]
+    copies = [torch.empty(shape, device="cuda") for _ in src]
+    with P.Sketch(3, 0, k, form) as sk:
+        go = sk.left if side == "left" else sk.right
+        want = [go(a).clone() for a in src]
+        torch.cuda.synchronize()
+        other = torch.cuda.Stream()
+
+        def steps():
+            here = torch.cuda.current_stream()
+            for a, y, c in zip(src, ys, copies):
+                other.wait_stream(here)
+                with torch.cuda.stream(other):
+                    torch.mul(a, 1.0, out=A)
+                here.wait_stream(other)
+                go(A, out=y)
+                other.wait_stream(here)
+                with torch.cuda.stream(other):
+                    c.copy_(y)
+                here.wait_stream(other)
+                go(src[0], out=y)
+
+        for y in ys + copies:
+            y.fill_(float("nan"))
+        torch.cuda.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                steps()
+            g.replay()
+        else:
+            steps()
+        torch.cuda.synchronize()
+        for y, c, w in zip(ys, copies, want):
+            assert torch.equal(c, w)
+            assert torch.equal(y, want[0])
+        assert sk.status() == 0
