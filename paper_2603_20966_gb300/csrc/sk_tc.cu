@@ -1221,14 +1221,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                            ig.pr->conv_inline && (DIST != kMixed || ig.dist == kRademacher);
         if ((!EC && !SRING) || wconv) {  // otherwise the A tile is certified by others
           // With a separate S ring a group is released NSS stages after its
-          // slot of S, and (behind an item whose A it did not wait for) the A
-          // tile of stage g - NSO may still be on its way: full_b is then a
-          // whole phase behind and the parity test below would let the group
-          // split a slot that holds another stage.  The MMAs of that stage
-          // come first; the copy awaited below started behind them, so this
-          // adds nothing to the wait (batch of 256: 4.86 ms).
+          // slot of S, and at its first stage of an item (behind one whose A
+          // it did not wait for) the A tile of stage g - NSO may still be on
+          // its way: full_b is then a whole phase behind and the parity test
+          // below would let the group split a slot that holds another stage.
+          // The MMAs of that stage come first; the copy awaited below started
+          // behind them, so this adds nothing to the wait.
+          static_assert(!SRING || C::NSO % C::NGROUPS == 0, "stage g - NSO is the group's own");
           const int v = g - C::NSO;
-          ok = !SRING || v < 0 || mbar_wait(empty_o(v % C::NSS), (v / C::NSS) & 1, ab, 0x47, g);
+          ok = !SRING || s >= C::NSO || v < 0 ||
+               mbar_wait(empty_o(v % C::NSS), (v / C::NSS) & 1, ab, 0x47, g);
           // this CTA's split A tile of the stage has landed
           ok = ok && mbar_wait(full_b(so), (g / C::NSO) & 1, ab, 0x40, g);
           if (!__all_sync(0xffffffffu, ok)) {
