@@ -335,7 +335,8 @@ sk_status sk_batch_destroy(sk_batch_handle b);
  *  - at each step boundary (one of its two compute streams idle) launches
  *    every admitted request not yet launched as one step: the SK_BF16X2
  *    requests as one persistent batched launch plus one batched reduce
- *    (as sk_batch_run), the SK_FP32 requests as fused SIMT launches.  Steps
+ *    (as sk_batch_run), the SK_FP32 requests as FP32 left sketches of their
+ *    own.  Steps
  *    on the two streams overlap on the device, so requests arriving while
  *    others run join the next step without waiting for the GPU to drain;
  *  - completes a step when its event is observed; the copy of A and the
@@ -426,7 +427,7 @@ sk_status sk_server_destroy(sk_server_handle s);
  * barrier: roles 1 TMA producer, 2 MMA issuer, 3 epilogue, 4 worker;
  * barriers 0 staging full, 1 staging empty, 2 operand full, 3 operand empty,
  * 4 accumulator full, 5 accumulator empty, 6 S rows received from another
- * CTA, 8 work-queue slot free, 9 work item published), [2] the pipeline stage (or
+ * CTA, 7 MMAs of the stage that had the A slot before, 8 work-queue slot free, 9 work item published), [2] the pipeline stage (or
  * accumulation chain) it was waiting for, [3] the linear index of its CTA.
  * Words 1-3 are meaningful only when word 0 is SK_ETIMEOUT. */
 sk_status sk_debug_status(sk_handle h, void* stream, int32_t out[4]);
