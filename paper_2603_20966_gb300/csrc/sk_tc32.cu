@@ -100,9 +100,9 @@ constexpr int SEEN = 4;         // items whose flags are kept at a time
 constexpr int REDO_BITS = 512;  // items (modulo this) that run a second time
 struct Seen {
   // columns 64 c + 2 l + x of an item's tile as bit l of word 2 c + x
-  uint32_t normal[SEEN][2 * NCH];  // an element of at least kSmall was seen
-  uint32_t small[SEEN][2 * NCH];   // a smaller one was, before any of those
-  uint32_t all[SEEN];              // normal elements were seen in every column
+  uint32_t normal[SEEN][2 * NCH];  // a warp that met small elements saw one of kSmall or more
+  uint32_t small[SEEN][2 * NCH];   // a warp saw smaller ones (not zeros) and none of those
+  uint32_t all[SEEN];              // a warp saw one of kSmall or more in every column
   uint32_t redo[REDO_BITS / 32];   // items with columns that may be small all through,
   uint32_t any_redo;               // and whether there are any
   uint32_t scaled[2 * NCH];        // columns that the second run multiplies by kUp
@@ -133,7 +133,6 @@ struct F32Params {
   int chain;  // stages per accumulation chain
   int cross;  // chains per accumulation of the cross terms
   int vec2;   // rows of A on 8-byte boundaries
-  int dist;
   PhiloxRoundKeys rk;
   int* status;
   uint64_t timeout_ns;
@@ -823,7 +822,6 @@ cudaError_t tc32_sketch_left(const sk_sketch* h, const GemmShape& s, const float
   p.chain = pl.chain;
   p.cross = pl.cross;
   p.vec2 = reinterpret_cast<uintptr_t>(A) % 8 == 0 && lda % 2 == 0;
-  p.dist = h->dist;
   p.rk = round_keys(make_key(h->seed));
   p.status = h->d_status;
   p.timeout_ns = h->wait_limit_ns;
